@@ -198,8 +198,16 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 // S_dev (optional): the count is read on the device, S is its upper bound
 int launch_make_atoms(const int32_t* idx, const float* x, int S, int N, double dl, float4* atoms,
                       cudaStream_t st, const int32_t* S_dev = nullptr);
+// Scales of the fixed-point w-term: turns x 2^32 = (w w_scale) (s s_scale) >> shift.
+struct PhaseScale {
+  float w_scale = 1.f, s_scale = 1.f;
+  int shift = 0;
+  bool fixed = false;   // the plan's w-term fits (else the double-float product)
+};
+PhaseScale phase_scale(double w_max, double s_max);   // bounds of |w| and of |n - 1|
 int launch_residual(const int4* vis_fx, const float2* V, int64_t M, const float4* atoms, int S,
-                    float2* out, double* sumsq, cudaStream_t st, const int32_t* S_dev = nullptr);
+                    float2* out, double* sumsq, const PhaseScale& sc, cudaStream_t st,
+                    const int32_t* S_dev = nullptr);
 int launch_gram(const int4* vis_fx, const float2* V, int64_t M, const float4* atomsA, int nA,
                 const float4* atomsB, int nB, bool with_v, double* acc, int ldacc,
                 cudaStream_t st, bool clear = true);
@@ -312,6 +320,7 @@ struct pc_plan_s {
   double fov = 0, dl = 0, beta = 0;
   double w0 = 0, dw = 1, s_c = 0, w_min = 0, w_max = 0;
   bool wstack = false;
+  pc::PhaseScale phase;   // fixed-point scales of the residual's w-term
   int grid_mode = 0;  // 0 auto, 1 CUDA cores, 2 tensor cores, 3 CUDA cores over plane
                       // windows (2 and 3: w-stacking only; else mode 1 runs)
   int grid_piece = 0; // gridding sub-problem size in slots (0: chosen for even waves)

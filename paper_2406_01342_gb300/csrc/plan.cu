@@ -621,6 +621,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   const double r2c = 2.0 * half * half;
   const double s_min = -r2c / (1.0 + std::sqrt(1.0 - r2c));
   const double s_max = 0.0;
+  p->phase = phase_scale(std::max(std::fabs(p->w_min), std::fabs(p->w_max)), -s_min);
   if (M > 0 && p->w_max > p->w_min) {
     p->wstack = true;
     p->dw = 1.0 / (2.0 * (s_max - s_min));

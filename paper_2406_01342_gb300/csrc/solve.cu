@@ -352,7 +352,7 @@ extern "C" int pc_forward_sparse(pc_plan_t p, const int32_t* idx, const float* x
   PC_TRY(p->atomsA.ensure(sizeof(float4) * std::max(S, 1)));
   PC_TRY(make_atoms_checked(idx, x, S, p->N, p->dl, p->atomsA.as<float4>(), p->iscal, st));
   PC_TRY(launch_residual(p->vis_fx, nullptr, p->M, p->atomsA.as<float4>(), S,
-                         reinterpret_cast<float2*>(y), nullptr, st));
+                         reinterpret_cast<float2*>(y), nullptr, p->phase, st));
   return PC_OK;
 }
 
@@ -437,7 +437,7 @@ extern "C" int pc_certificate(pc_plan_t p, const pc_c32* V, const int32_t* idx, 
   PC_CUDA(cudaMemsetAsync(p->dscal, 0, sizeof(double), st));
   PC_CUDA(cudaMemsetAsync(p->uscal, 0, 2 * sizeof(unsigned), st));
   PC_TRY(launch_residual(p->vis_fx, reinterpret_cast<const float2*>(V), p->M,
-                         p->atomsA.as<float4>(), S, p->resid, p->dscal, st));
+                         p->atomsA.as<float4>(), S, p->resid, p->dscal, p->phase, st));
   PC_TRY(adjoint_grid_impl(p, p->resid, mu, (float)(1.0 / lambda), p->uscal, st));
   if (mu_inf_host || sumsq_host) {
     unsigned b = 0;
@@ -639,7 +639,7 @@ int SolveJob::start(pc_plan_s* plan, const float2* V_dev, double lambda_, double
   // flag cleared (the gridding flag iscal[7] may still report an earlier call)
   PC_CUDA(cudaMemsetAsync(p->iscal, 0, 7 * sizeof(int32_t), st));
   PC_CUDA(cudaMemsetAsync(p->dscal, 0, 2 * sizeof(double), st));
-  PC_TRY(launch_residual(p->vis_fx, V, p->M, nullptr, 0, p->resid, p->dscal, st));
+  PC_TRY(launch_residual(p->vis_fx, V, p->M, nullptr, 0, p->resid, p->dscal, p->phase, st));
   rb->hd[1] = (c.rule == 1 && c.lmax > 0) ? (1.0 - delta) * c.lmax : -1.0;   // Delta of rule R1
   PC_CUDA(cudaMemcpyAsync(p->dscal + 4, &rb->hd[1], sizeof(double), cudaMemcpyHostToDevice, st));
   PC_CUDA(cudaMemcpyAsync(&rb->hd[0], p->dscal, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -728,8 +728,8 @@ int SolveJob::enqueue_chain(int bound, int warm_S) {
                                   p->atom_tab);
     PC_LAUNCH_CHECK();
   }
-  PC_TRY(launch_residual(p->vis_fx, V, p->M, p->atomsA.as<float4>(), bound, p->resid, p->dscal, st,
-                         n_sup_dev));
+  PC_TRY(launch_residual(p->vis_fx, V, p->M, p->atomsA.as<float4>(), bound, p->resid, p->dscal, p->phase,
+                         st, n_sup_dev));
   PC_CUDA(cudaMemsetAsync(p->uscal, 0, 2 * sizeof(unsigned), st));
   PC_TRY(adjoint_grid_impl(p, p->resid, mu_dst, (float)(1.0 / lambda), p->uscal, st));
   PC_TRY(explore());

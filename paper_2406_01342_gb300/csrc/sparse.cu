@@ -10,6 +10,8 @@
 // Phases are generated on the fly: the lattice part i' U_k + j' V_k in exact
 // 32-bit fixed-point turns, the w-term as a double-float product, one FP32
 // sincospi per (visibility, atom) pair.
+#include <cmath>
+
 #include "pc_internal.cuh"
 
 namespace pc {
@@ -26,11 +28,129 @@ __global__ void k_make_atoms(const int32_t* __restrict__ idx, const float* __res
   atoms[s] = make_atom(p, x ? x[s] : 1.f, x != nullptr, N, dl);
 }
 
-constexpr int RES_CHUNK = 1024;
+constexpr int RES_CHUNK = 1024;  // atoms in shared memory (16 KB)
+
+// Fixed-point w: w_hi + w_lo in units of 1 / scale (each term rounded, the
+// larger one exact).
+__device__ __forceinline__ int fixed32(float hi, float lo, float scale) {
+  return __float2int_rn(hi * scale) + __float2int_rn(lo * scale);
+}
 
 // out = V - Phi_S x  (or Phi_S x when V is null); sumsq += ||out||^2 in float64.
+//
+// The phase i' U + j' V + w s of a (visibility, atom) pair stays in 32-bit
+// fixed-point turns: w and s = n - 1 are 32-bit integers at power-of-two scales
+// (PhaseScale), the 64-bit product is shifted to turns, and the sum wraps, which
+// is the exact reduction. Its top bit is the sign of a half turn, taken onto the
+// weight; the next 23 become the mantissa of a float in [1, 2), that is an angle
+// in [-pi/2, pi/2] to 2^-25 turns, where the fast sine and cosine are accurate to
+// 4e-7.
+//
+// What bounds it: the two MUFU operations a phase, 16 a cycle and SM, so 8
+// phases a cycle. The double-float w-term with two roundings to the nearest turn
+// and an integer conversion (which shares that pipe) issued 24 instructions and
+// ran 4.1 phases a cycle; this is 12 instructions, none of them a conversion.
+//
+// A block's eight warps hold GROUPS groups, each summing its share of the atoms
+// for the same 256 / GROUPS x VPT visibilities, so that few visibilities still
+// fill the SMs; the group sums meet in shared memory.
+template <int VPT, int GROUPS>
 __global__ void __launch_bounds__(256)
 k_residual(const int4* __restrict__ vis, const float2* __restrict__ V, int64_t M,
+           const float4* __restrict__ atoms, int S, float2* __restrict__ out,
+           double* __restrict__ sumsq, const int32_t* __restrict__ S_dev, PhaseScale sc) {
+  constexpr int LANES = 256 / GROUPS;                 // visibilities side by side
+  __shared__ int4 sa[RES_CHUNK];                      // {i', j', s, x / n}
+  __shared__ float2 part[GROUPS > 1 ? GROUPS - 1 : 1][VPT][GROUPS > 1 ? LANES : 1];
+  __shared__ double red[8];
+  if (S_dev) S = min(S, *S_dev);
+  const int tid = threadIdx.x, group = tid / LANES, at_lane = tid % LANES;
+  const int64_t k0 = blockIdx.x * (int64_t)(VPT * LANES) + at_lane;   // visibility j: k0 + LANES j
+  int u[VPT], v[VPT], w[VPT];
+  float ar[VPT], ai[VPT];
+#pragma unroll
+  for (int j = 0; j < VPT; ++j) {
+    const int64_t k = k0 + LANES * j;
+    const int4 q = k < M ? vis[k] : make_int4(0, 0, 0, 0);
+    u[j] = q.x;
+    v[j] = q.y;
+    w[j] = fixed32(__int_as_float(q.z), __int_as_float(q.w), sc.w_scale);
+    ar[j] = ai[j] = 0.f;
+  }
+  // a quarter turn, so that the top bit tells the half, and the rounding of the shift by 8
+  const long long bias = (long long)(0x40000000u + 128u) << sc.shift;
+  for (int s0 = 0; s0 < S; s0 += RES_CHUNK) {
+    const int cnt = min(RES_CHUNK, S - s0);
+    for (int t = tid; t < cnt; t += 256) {
+      const float4 at = atoms[s0 + t];
+      const int packed = __float_as_int(at.x);
+      sa[t] = make_int4(packed >> 16, (int)(short)(packed & 0xffff), fixed32(at.y, at.z, sc.s_scale),
+                        __float_as_int(at.w));
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int t = group; t < cnt; t += GROUPS) {
+      const int4 at = sa[t];
+#pragma unroll
+      for (int j = 0; j < VPT; ++j) {
+        const long long ws = (long long)w[j] * at.z + bias;
+        const unsigned th = (unsigned)at.x * (unsigned)u[j] + ((unsigned)at.y * (unsigned)v[j] +
+                            __funnelshift_r((unsigned)ws, (unsigned)((unsigned long long)ws >> 32), sc.shift));
+        const float f = __uint_as_float(((th >> 8) & 0x7fffffu) | 0x3f800000u);
+        const float x = __int_as_float(at.w ^ (int)(th & 0x80000000u));
+        float sn, cs;
+        __sincosf(fmaf(f, 3.14159265358979f, -4.71238898038469f), &sn, &cs);
+        ar[j] = fmaf(x, cs, ar[j]);
+        ai[j] = fmaf(-x, sn, ai[j]);
+      }
+    }
+    __syncthreads();
+  }
+  if (GROUPS > 1) {
+    if (group > 0)
+#pragma unroll
+      for (int j = 0; j < VPT; ++j) part[group - 1][j][at_lane] = make_float2(ar[j], ai[j]);
+    __syncthreads();
+    if (group == 0)
+#pragma unroll
+      for (int j = 0; j < VPT; ++j)
+        for (int q = 0; q < GROUPS - 1; ++q) {
+          ar[j] += part[q][j][at_lane].x;
+          ai[j] += part[q][j][at_lane].y;
+        }
+  }
+  double local = 0.0;
+  if (group == 0) {
+#pragma unroll
+    for (int j = 0; j < VPT; ++j) {
+      const int64_t k = k0 + LANES * j;
+      if (k < M) {
+        float2 r = make_float2(ar[j], ai[j]);
+        if (V) {
+          const float2 q = V[k];
+          r = make_float2(q.x - ar[j], q.y - ai[j]);
+        }
+        out[k] = r;
+        local += (double)r.x * r.x + (double)r.y * r.y;
+      }
+    }
+  }
+  if (sumsq) {
+    for (int off = 16; off; off >>= 1) local += __shfl_xor_sync(0xffffffffu, local, off);
+    if ((tid & 31) == 0) red[tid >> 5] = local;
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int q = 0; q < 8; ++q) t += red[q];
+      atomicAdd(sumsq, t);
+    }
+  }
+}
+
+// The same with the w-term as a double-float product (phase_turns), for plans
+// whose w-term spans more turns than a 32-bit fixed-point phase resolves.
+__global__ void __launch_bounds__(256)
+k_residual_wide(const int4* __restrict__ vis, const float2* __restrict__ V, int64_t M,
            const float4* __restrict__ atoms, int S, float2* __restrict__ out,
            double* __restrict__ sumsq, const int32_t* __restrict__ S_dev) {
   __shared__ float4 sa[RES_CHUNK];
@@ -354,12 +474,44 @@ int make_atoms_checked(const int32_t* idx, const float* x, int S, int N, double 
   return PC_OK;
 }
 
+PhaseScale phase_scale(double w_max, double s_max) {
+  // |w| scale and |s| scale below 2^30, their product at most 2^63
+  auto fit = [](double m) { return m > 0.0 ? 30 - (int)std::floor(std::log2(m)) - 1 : 0; };
+  const int a = std::min(std::max(fit(w_max), -90), 90);
+  const int b = std::min(std::min(std::max(fit(s_max), -90), 90), 63 - a);
+  PhaseScale sc;
+  sc.w_scale = std::ldexp(1.f, a);
+  sc.s_scale = std::ldexp(1.f, b);
+  sc.shift = a + b - 32;
+  sc.fixed = w_max * s_max <= 32.0 && sc.shift >= 0 && sc.shift <= 31;
+  return sc;
+}
+
+// The fixed-point kernel wherever the w-term stays within 32 turns (its 32-bit
+// factors then leave it 1.5e-8 turns; the configurations have 0.2 to 4), else the
+// double-float one. Visibilities per block by their number, so that there are two
+// blocks or more an SM (200k visibilities x 200 atoms: 44 us in blocks of 512).
 int launch_residual(const int4* vis_fx, const float2* V, int64_t M, const float4* atoms, int S,
-                    float2* out, double* sumsq, cudaStream_t st, const int32_t* S_dev) {
+                    float2* out, double* sumsq, const PhaseScale& sc, cudaStream_t st, const int32_t* S_dev) {
   ProfScope prof_scope_(PROF_RESIDUAL, st);
   if (M <= 0) return PC_OK;
   prof_scope_.kernels = 1;
-  k_residual<<<ceil_div(M, 256), 256, 0, st>>>(vis_fx, V, M, atoms, S, out, sumsq, S_dev);
+#define PC_RESIDUAL(VPT, GROUPS)                                                                              \
+  k_residual<VPT, GROUPS><<<ceil_div(M, VPT * 256 / GROUPS), 256, 0, st>>>(vis_fx, V, M, atoms, S, out, sumsq, \
+                                                                           S_dev, sc)
+  if (!sc.fixed)
+    k_residual_wide<<<ceil_div(M, 256), 256, 0, st>>>(vis_fx, V, M, atoms, S, out, sumsq, S_dev);
+  else if (M >= 1000000)
+    PC_RESIDUAL(4, 1);
+  else if (M >= 400000)
+    PC_RESIDUAL(2, 1);
+  else if (M >= 100000)
+    PC_RESIDUAL(2, 2);
+  else if (M >= 40000)
+    PC_RESIDUAL(1, 2);
+  else
+    PC_RESIDUAL(1, 8);
+#undef PC_RESIDUAL
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
