@@ -270,8 +270,12 @@ k_degrid(const int4* __restrict__ subs, const int2* __restrict__ slot_vis, const
 // "degrid_fft"; the interpolation is timed as "degrid".
 static int degrid_ffts(pc_plan_s* p, const float* img, cudaStream_t st) {
   ProfScope prof_scope_(PROF_DEGRID_FFT, st);
-  const int N = p->N, G = p->G, n_act = p->n_active_rows;
+  const int N = p->Nt, G = p->G, n_act = p->n_active_rows;
   const int ws = p->wstack ? 1 : 0;
+  if (p->resample.K > 0) {
+    PC_TRY(launch_downsample(p, img, st));
+    img = p->small_img;
+  }
   if (fft_big_size(G) && p->fft_warp != 0) {
     // one-CTA transforms (fft_big.cu) for G = 2048 .. 8192
     PC_TRY(launch_degrid_ffts_big(p, img, st));
@@ -336,7 +340,7 @@ static int degrid_ffts(pc_plan_s* p, const float* img, cudaStream_t st) {
   }
   }
   }
-  prof_scope_.kernels = 2;
+  prof_scope_.kernels = p->resample.K > 0 ? 4 : 2;
   return PC_OK;
 }
 

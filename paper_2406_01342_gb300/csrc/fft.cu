@@ -338,11 +338,11 @@ int launch_fft_rows(pc_plan_s* p, cudaStream_t st) {
     if (p->G == 1024) {
       static bool done = false;
       PC_TRY(allow_smem(k_fft_rows_w<32>, done));
-      k_fft_rows_w<32><<<grid, 256, smem, st>>>(p->grid, p->fft1, p->N, p->tw2, p->active_rows, p->col_mask);
+      k_fft_rows_w<32><<<grid, 256, smem, st>>>(p->grid, p->fft1, p->Nt, p->tw2, p->active_rows, p->col_mask);
     } else {
       static bool done = false;
       PC_TRY(allow_smem(k_fft_rows_w<16>, done));
-      k_fft_rows_w<16><<<grid, 256, smem, st>>>(p->grid, p->fft1, p->N, p->tw2, p->active_rows, p->col_mask);
+      k_fft_rows_w<16><<<grid, 256, smem, st>>>(p->grid, p->fft1, p->Nt, p->tw2, p->active_rows, p->col_mask);
     }
     PC_LAUNCH_CHECK();
     return PC_OK;
@@ -361,7 +361,7 @@ int launch_fft_rows(pc_plan_s* p, cudaStream_t st) {
   }
   dim3 grid(p->n_active_rows / R, p->P);
   prof_scope_.kernels = 1;
-  k_fft_rows<<<grid, 256, smem, st>>>(p->grid, p->fft1, p->G, p->logG, p->N, R, p->twiddle,
+  k_fft_rows<<<grid, 256, smem, st>>>(p->grid, p->fft1, p->G, p->logG, p->Nt, R, p->twiddle,
                                       p->active_rows);
   PC_LAUNCH_CHECK();
   return PC_OK;
@@ -376,12 +376,11 @@ int cols_planes_per_pass(const pc_plan_s* p) {
   return std::max(pg, 1);
 }
 
-int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
-                             cudaStream_t st) {
-  ProfScope prof_scope_(PROF_FFT_COLS, st);
+static int cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits, cudaStream_t st,
+                         ProfScope& prof_scope_) {
   if (fft_cols_big(p)) {
     if (p->n_active_rows == 0) {                // nothing reaches the grid: mu = 0
-      PC_CUDA(cudaMemsetAsync(mu, 0, sizeof(float) * (size_t)p->N * p->N, st));
+      PC_CUDA(cudaMemsetAsync(mu, 0, sizeof(float) * (size_t)p->Nt * p->Nt, st));
       return PC_OK;
     }
     prof_scope_.kernels = 1;
@@ -394,14 +393,14 @@ int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* max
     const int ws = p->wstack ? 1 : 0;
     const bool one = wpr == p->P;                  // every warp exactly one plane
     // turns of the CTA's rows; with several planes per warp also 8 running sums of N
-    const size_t smem = warp_fft_smem(p->G, one ? (ws ? rpc * p->N : 0) : rpc * p->N + 8 * p->N);
+    const size_t smem = warp_fft_smem(p->G, one ? (ws ? rpc * p->Nt : 0) : rpc * p->Nt + 8 * p->Nt);
     prof_scope_.kernels = 1;
-    const unsigned nb = (unsigned)ceil_div(p->N, rpc);
+    const unsigned nb = (unsigned)ceil_div(p->Nt, rpc);
 #define PC_COLS_W(LL, ONE)                                                                        \
   {                                                                                               \
     static bool done = false;                                                                     \
     PC_TRY(allow_smem(k_fft_cols_w<LL, ONE>, done));                                              \
-    k_fft_cols_w<LL, ONE><<<nb, 256, smem, st>>>(p->fft1, p->pix_tab, mu, p->N, p->P, wpr, ws,   \
+    k_fft_cols_w<LL, ONE><<<nb, 256, smem, st>>>(p->fft1, p->pix_tab, mu, p->Nt, p->P, wpr, ws,   \
                                                  p->tw2, p->row_mask, scale, maxbits);            \
   }
     if (p->G == 1024) {
@@ -415,7 +414,7 @@ int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* max
   }
   const int PG = cols_planes_per_pass(p);
   const size_t smem = ((size_t)2 * PG * p->G + p->G) * sizeof(float2);
-  const int jpt = (p->N + 255) / 256;
+  const int jpt = (p->Nt + 255) / 256;
   prof_scope_.kernels = 1;
   const int ws = p->wstack ? 1 : 0;
 #define PC_COLS_CASE(J)                                                                         \
@@ -426,7 +425,7 @@ int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* max
                                    200 * 1024));                                                \
       attr_set = true;                                                                          \
     }                                                                                           \
-    k_fft_cols<J><<<p->N, 256, smem, st>>>(p->fft1, p->pix_tab, mu, p->G, p->logG, p->N, p->P,  \
+    k_fft_cols<J><<<p->Nt, 256, smem, st>>>(p->fft1, p->pix_tab, mu, p->G, p->logG, p->Nt, p->P,  \
                                            PG, ws, p->twiddle, scale, maxbits);                 \
     break;                                                                                      \
   }
@@ -440,11 +439,20 @@ int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* max
     case 9: case 10: case 11: case 12: case 13: case 14: case 15:
     PC_COLS_CASE(16)
     default:
-      return fail(PC_ERR_INVALID_ARG, "fft: image side %d too large", p->N);
+      return fail(PC_ERR_INVALID_ARG, "fft: image side %d too large", p->Nt);
   }
 #undef PC_COLS_CASE
   PC_LAUNCH_CHECK();
   return PC_OK;
+}
+
+int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
+                             cudaStream_t st) {
+  ProfScope prof_scope_(PROF_FFT_COLS, st);
+  if (p->resample.K == 0) return cols_epilogue(p, mu, scale, maxbits, st, prof_scope_);
+  PC_TRY(cols_epilogue(p, p->small_img, 1.0f, nullptr, st, prof_scope_));
+  prof_scope_.kernels += 2;
+  return launch_upsample(p, mu, scale, maxbits, st);
 }
 
 }  // namespace pc

@@ -357,7 +357,7 @@ int compact_blocks(const pc_plan_s* p) { return ceil_div(std::max(p->n_active_ro
 
 int launch_fft_rows_big(pc_plan_s* p, cudaStream_t st) {
   const int nb = compact_blocks(p);
-  PC_TRY(p->xc.ensure(sizeof(float2) * (size_t)p->P * nb * p->N * 4));
+  PC_TRY(p->xc.ensure(sizeof(float2) * (size_t)p->P * nb * p->Nt * 4));
   float2* Xc = p->xc.as<float2>();
 #define PC_ROWS(RR)                                                                                        \
   const size_t smem = sizeof(float2) * cfft::Cfg<RR>::Z_ELEMS;                                             \
@@ -366,7 +366,7 @@ int launch_fft_rows_big(pc_plan_s* p, cudaStream_t st) {
     PC_TRY(allow(k_fft_rows_big<RR>, smem));                                                               \
     done = true;                                                                                           \
   }                                                                                                        \
-  k_fft_rows_big<RR><<<dim3(p->n_active_rows, p->P), 32 * RR, smem, st>>>(p->grid, Xc, p->N, nb,           \
+  k_fft_rows_big<RR><<<dim3(p->n_active_rows, p->P), 32 * RR, smem, st>>>(p->grid, Xc, p->Nt, nb,           \
                                                                            p->active_rows, p->col_bits,    \
                                                                            p->tw_big, p->tw_in);
   PC_BIG_DISPATCH(p->G, PC_ROWS)
@@ -397,8 +397,8 @@ int make_xc_tensor_map(pc_plan_s* p) {
     }
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  const cuuint64_t dims[2] = {(cuuint64_t)8 * p->N, (cuuint64_t)p->P * nb};
-  const cuuint64_t strides[1] = {(cuuint64_t)8 * p->N * sizeof(float)};
+  const cuuint64_t dims[2] = {(cuuint64_t)8 * p->Nt, (cuuint64_t)p->P * nb};
+  const cuuint64_t strides[1] = {(cuuint64_t)8 * p->Nt * sizeof(float)};
   const cuuint32_t box[2] = {8, (cuuint32_t)p->xmap_by};
   const cuuint32_t elem[2] = {1, 1};
   const CUresult r = encode(&p->xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p->xc.p, dims, strides, box, elem,
@@ -413,7 +413,7 @@ int launch_fft_cols_big(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
   const int ws = p->wstack ? 1 : 0;
   const size_t stage = cols_stage_bytes(p->xmap_boxes, p->xmap_by);
   const bool restricted = p->n_img_rows > 0;
-  const int rows_img = restricted ? p->n_img_rows : p->N;
+  const int rows_img = restricted ? p->n_img_rows : p->Nt;
   const int* list = restricted ? p->img_rows : nullptr;
 #define PC_COLS(RR)                                                                                        \
   const size_t smem = cols_z_bytes<RR>() + 2 * stage;                                                      \
@@ -425,7 +425,7 @@ int launch_fft_cols_big(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
     done = true;                                                                                           \
   }                                                                                                        \
   k_fft_cols_big<RR><<<rows_img, 32 * RR, smem, st>>>(p->xmap, p->xmap_boxes, p->xmap_by, p->pix_tab, mu,     \
-                                                     p->N, p->P, nb, ws, p->row_pos, p->tw_big, p->tw_in,   \
+                                                     p->Nt, p->P, nb, ws, p->row_pos, p->tw_big, p->tw_in,   \
                                                      scale, maxbits, p->iscal + 7, list);
   PC_BIG_DISPATCH(p->G, PC_COLS)
 #undef PC_COLS
@@ -436,11 +436,11 @@ int launch_fft_cols_big(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
 // The degridding's two FFT passes: img (N x N) -> grid_q[b][.] at the reachable rows.
 int launch_degrid_ffts_big(pc_plan_s* p, const float* img, cudaStream_t st) {
   const int nb = compact_blocks(p);
-  PC_TRY(p->xc.ensure(sizeof(float2) * (size_t)p->P * nb * p->N * 4));
+  PC_TRY(p->xc.ensure(sizeof(float2) * (size_t)p->P * nb * p->Nt * 4));
   float2* Xc = p->xc.as<float2>();
   const int ws = p->wstack ? 1 : 0;
   const bool restricted = p->n_img_rows > 0;
-  const int rows_img = restricted ? p->n_img_rows : p->N;
+  const int rows_img = restricted ? p->n_img_rows : p->Nt;
   const int* list = restricted ? p->img_rows : nullptr;
   const uint32_t* bits = restricted ? p->img_row_bits : nullptr;
 #define PC_DG(RR)                                                                                          \
@@ -451,12 +451,12 @@ int launch_degrid_ffts_big(pc_plan_s* p, const float* img, cudaStream_t st) {
     PC_TRY(allow(k_degrid_rows_big<RR>, smem));                                                            \
     done = true;                                                                                           \
   }                                                                                                        \
-  k_degrid_cols_big<RR><<<rows_img, 32 * RR, smem, st>>>(img, p->pix_tab, p->N, p->P, nb,                 \
+  k_degrid_cols_big<RR><<<rows_img, 32 * RR, smem, st>>>(img, p->pix_tab, p->Nt, p->P, nb,                 \
                                                         p->n_active_rows, ws, p->row_pos, p->active_rows,   \
                                                         p->tw_big, p->tw_in, Xc, list);                    \
   PC_LAUNCH_CHECK();                                                                                       \
   k_degrid_rows_big<RR><<<dim3(p->n_active_rows, p->P), 32 * RR, smem, st>>>(                              \
-      Xc, p->N, nb, p->active_rows, p->col_bits, p->tw_big, p->tw_in, p->grid, bits);
+      Xc, p->Nt, nb, p->active_rows, p->col_bits, p->tw_big, p->tw_in, p->grid, bits);
   PC_BIG_DISPATCH(p->G, PC_DG)
 #undef PC_DG
   PC_LAUNCH_CHECK();

@@ -255,12 +255,12 @@ k_grid_win(const int4* __restrict__ subs, const int* __restrict__ win_off, const
 
 }  // namespace
 
-// Mode 3, or the default (mode 0) on grids of side 2048 and more, where it
+// Mode 3, or the default (mode 0) for images with grids of side 2048 and more, where it
 // measured faster than the tensor-core gridding (2048^2 / 2M: 0.81 against
 // 1.31 ms; 4096^2 / 10M: 2.8 against 4.9 ms; at 512^2 / 200k the tensor cores
 // win, 0.10 against 0.15 ms).
 bool grid_win_mode(const pc_plan_s* p) {
-  return p->wstack && p->W <= 7 && p->Pw <= GW_MAXW && (p->grid_mode == 3 || (p->grid_mode == 0 && p->G >= 2048));
+  return p->wstack && p->W <= 7 && p->Pw <= GW_MAXW && (p->grid_mode == 3 || (p->grid_mode == 0 && p->G_image >= 2048));
 }
 
 int launch_grid_win(pc_plan_s* p, const float2* h, cudaStream_t st) {

@@ -299,6 +299,22 @@ int launch_fft_rows_big(pc_plan_s* p, cudaStream_t st);
 int launch_fft_cols_big(pc_plan_s* p, float* mu, float scale, unsigned* maxbits, cudaStream_t st);
 int launch_degrid_ffts_big(pc_plan_s* p, const float* img, cudaStream_t st);
 int make_xc_tensor_map(pc_plan_s* p);   // after xc is allocated
+// resample.cu: transforms on a smaller image of the same field
+struct Resample {
+  int K = 0;            // interpolation taps (0: the transforms run on the image itself)
+  int Nt = 0, G = 0;    // side of the transforms' image and of their grid
+  double d = 1.0, beta = 0.0;
+};
+struct BandTable {
+  int* first = nullptr;
+  float* w = nullptr;
+  int width = 0;
+};
+Resample choose_resample(int N, int G, double turns);
+void resample_widths(const Resample& r, int N, int* up, int* down);
+int fill_band_tables(const Resample& r, int N, BandTable* up, BandTable* down, cudaStream_t st);
+int launch_upsample(pc_plan_s* p, float* img, float scale, unsigned* maxbits, cudaStream_t st);
+int launch_downsample(pc_plan_s* p, const float* img, cudaStream_t st);
 // degrid.cu: y = Phi(img) for a dense N x N image (type-2 NUFFT), y cleared first
 int forward_grid_impl(pc_plan_s* p, const float* img, float2* y, cudaStream_t st);
 
@@ -310,7 +326,13 @@ struct pc_plan_s {
   int device = 0;
   int64_t M = 0;
   int N = 0;          // image side
-  int G = 0;          // oversampled grid side (power of two >= 2N)
+  int G_image = 0;    // oversampled grid side of the image (power of two >= 2N)
+  int G = 0;          // grid side of the transforms: G_image, or smaller with their smaller image
+  int Nt = 0;         // image side of the transforms: N, or G / 2 (resample.K > 0)
+  pc::Resample resample;
+  pc::BandTable up, down;        // resample.K > 0: interpolation to the N x N pixels and its transpose
+  float* small_img = nullptr;    // Nt x Nt
+  float* small_tmp = nullptr;    // Nt x N, between the two applications
   int logG = 0;
   int T = 32;         // gridding tile side
   int nT = 0;         // tiles per side = G / T

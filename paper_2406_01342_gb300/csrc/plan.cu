@@ -81,8 +81,9 @@ __device__ __forceinline__ unsigned long long ordered_bits(double d) {
 }
 
 __global__ void k_uvw_scan(const double* __restrict__ uvw, int64_t M,
-                           unsigned long long* wmin, unsigned long long* wmax, int* bad) {
-  unsigned long long lo = ~0ull, hi = 0ull;
+                           unsigned long long* wmin, unsigned long long* wmax, unsigned long long* uvmax,
+                           int* bad) {
+  unsigned long long lo = ~0ull, hi = 0ull, uv = 0ull;
   int nonfinite = 0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < M;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -91,17 +92,23 @@ __global__ void k_uvw_scan(const double* __restrict__ uvw, int64_t M,
     unsigned long long o = ordered_bits(w);
     lo = o < lo ? o : lo;
     hi = o > hi ? o : hi;
+    // largest |u|, |v| (the bits of non-negative doubles order as integers)
+    const unsigned long long m = (unsigned long long)__double_as_longlong(fmax(fabs(u), fabs(v)));
+    uv = m > uv ? m : uv;
   }
   for (int off = 16; off; off >>= 1) {
     unsigned long long a = __shfl_xor_sync(0xffffffffu, lo, off);
     unsigned long long b = __shfl_xor_sync(0xffffffffu, hi, off);
     lo = a < lo ? a : lo;
     hi = b > hi ? b : hi;
+    const unsigned long long c = __shfl_xor_sync(0xffffffffu, uv, off);
+    uv = c > uv ? c : uv;
     nonfinite |= __shfl_xor_sync(0xffffffffu, nonfinite, off);
   }
   if ((threadIdx.x & 31) == 0) {
     atomicMin(wmin, lo);
     atomicMax(wmax, hi);
+    atomicMax(uvmax, uv);
     if (nonfinite) atomicOr(bad, 1);
   }
 }
@@ -110,7 +117,8 @@ __global__ void k_uvw_scan(const double* __restrict__ uvw, int64_t M,
 // ordered by their tile-local row start b0 (then ps & 1). A sort key is
 // bin << 7 | (b0 + 8) << 1 | (ps & 1), b0 in [-(W - 1), T - 1].
 struct BinGeom {
-  double dl, w0, dw, s_c;
+  double dl, w0, dw, s_c;   // dl: pixel of the transforms' image
+  double dl_pix;            // pixel of the image (the phases of atoms)
   int G, T, nT, W, P;
   int Pw;           // plane-start pairs (plane windows): ((P - W) >> 1) + 1, or 1 without w-stacking
   unsigned nbins;   // tiles x Pw
@@ -120,11 +128,12 @@ constexpr int kBinSubBits = 7;
 __device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 // Grid coordinate in cells of a baseline component: frac(u dl) G in [0, G).
-__device__ __forceinline__ double grid_coord(double u, double dl, int G, double* frac_out) {
-  double U = u * dl;
-  double f = U - rint(U);
-  *frac_out = f;
-  double g = f * G;
+__device__ __forceinline__ double turn_frac(double u, double dl) {
+  const double U = u * dl;
+  return U - rint(U);
+}
+__device__ __forceinline__ double grid_coord(double u, double dl, int G) {
+  double g = turn_frac(u, dl) * G;
   if (g < 0.0) g += G;
   if (g >= G) g -= G;
   return g;
@@ -138,12 +147,11 @@ __global__ void k_vis_prep(const double* __restrict__ uvw, int64_t M, BinGeom g,
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= M) return;
   double u = uvw[3 * k], v = uvw[3 * k + 1], w = uvw[3 * k + 2];
-  double fu, fv;
-  double gu = grid_coord(u, g.dl, g.G, &fu);
-  double gv = grid_coord(v, g.dl, g.G, &fv);
+  double gu = grid_coord(u, g.dl, g.G);
+  double gv = grid_coord(v, g.dl, g.G);
   // 32-bit fixed-point turns of u dl and v dl (two's complement wrap = mod 1)
-  int Ufx = (int)(unsigned)(long long)llrint(fu * 4294967296.0);
-  int Vfx = (int)(unsigned)(long long)llrint(fv * 4294967296.0);
+  int Ufx = (int)(unsigned)(long long)llrint(turn_frac(u, g.dl_pix) * 4294967296.0);
+  int Vfx = (int)(unsigned)(long long)llrint(turn_frac(v, g.dl_pix) * 4294967296.0);
   float w_hi = (float)w;
   float w_lo = (float)(w - (double)w_hi);
   vis_fx[k] = make_int4(Ufx, Vfx, __float_as_int(w_hi), __float_as_int(w_lo));
@@ -281,9 +289,8 @@ __global__ void k_slot_gather(const double* __restrict__ uvw, const unsigned* __
   int64_t k = id >> 2;
   int c = id & 3;
   double u = uvw[3 * k], v = uvw[3 * k + 1], w = uvw[3 * k + 2];
-  double fu, fv;
-  double gu = grid_coord(u, g.dl, g.G, &fu);
-  double gv = grid_coord(v, g.dl, g.G, &fv);
+  double gu = grid_coord(u, g.dl, g.G);
+  double gv = grid_coord(v, g.dl, g.G);
   int a0 = (int)ceil(gu - 0.5 * g.W);
   int b0 = (int)ceil(gv - 0.5 * g.W);
   int ta = floor_div(a0, g.T) + (c & 1);
@@ -580,20 +587,21 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   TmpBufs tmp;
   tmp.st = st;
 
-  // ---- w range and finiteness
+  // ---- w range, largest |u|, |v| and finiteness
+  double uv_max = 0.0;
   if (M > 0) {
     unsigned long long* dmm;
     int* dbad;
-    PC_TRY(tmp.alloc((void**)&dmm, 2 * sizeof(unsigned long long) + sizeof(int) * 2));
-    dbad = reinterpret_cast<int*>(dmm + 2);
-    unsigned long long init[2] = {~0ull, 0ull};
+    PC_TRY(tmp.alloc((void**)&dmm, 3 * sizeof(unsigned long long) + sizeof(int) * 2));
+    dbad = reinterpret_cast<int*>(dmm + 3);
+    unsigned long long init[3] = {~0ull, 0ull, 0ull};
     int zero[2] = {0, 0};
     PC_CUDA(cudaMemcpyAsync(dmm, init, sizeof(init), cudaMemcpyHostToDevice, st));
     PC_CUDA(cudaMemcpyAsync(dbad, zero, sizeof(zero), cudaMemcpyHostToDevice, st));
     int blocks = (int)std::min<int64_t>(4096, (M + 255) / 256);
-    k_uvw_scan<<<blocks, 256, 0, st>>>(uvw, M, dmm, dmm + 1, dbad);
+    k_uvw_scan<<<blocks, 256, 0, st>>>(uvw, M, dmm, dmm + 1, dmm + 2, dbad);
     PC_LAUNCH_CHECK();
-    unsigned long long hmm[2];
+    unsigned long long hmm[3];
     int hbad[2];
     PC_CUDA(cudaMemcpyAsync(hmm, dmm, sizeof(hmm), cudaMemcpyDeviceToHost, st));
     PC_CUDA(cudaMemcpyAsync(hbad, dbad, sizeof(hbad), cudaMemcpyDeviceToHost, st));
@@ -607,17 +615,40 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
     };
     p->w_min = unmap(hmm[0]);
     p->w_max = unmap(hmm[1]);
+    std::memcpy(&uv_max, &hmm[2], sizeof(uv_max));
   }
 
   // ---- geometry
-  p->G = 32;
-  while (p->G < 2 * N) p->G *= 2;
+  p->G_image = 32;
+  while (p->G_image < 2 * N) p->G_image *= 2;
+  p->dl = p->fov / N;
+  p->Nt = N;
+  p->G = p->G_image;
+  {
+    // corner of the image; the transforms' smaller one reaches a little further
+    const double half = 0.5 * N * p->dl, r2 = 2.0 * half * half;
+    const double w_abs = std::max(std::fabs(p->w_min), std::fabs(p->w_max));
+    // turns per pixel: the baseline, and the slope |w| l / n of the w-term
+    const double turns = p->dl * (uv_max + w_abs * half / std::sqrt(1.0 - std::min(r2, 0.99)));
+    if (M > 0 && p->fft_warp != 0 && r2 < 0.4) p->resample = choose_resample(N, p->G_image, turns);
+    if (p->resample.K > 0) {
+      // its wider field takes more w-planes: not beyond the caller's cap
+      const double h = 0.5 * p->resample.Nt * p->dl * p->resample.d, r2t = 2.0 * h * h;
+      const double s_range = r2t / (1.0 + std::sqrt(1.0 - r2t));
+      if (std::ceil((p->w_max - p->w_min) * 2.0 * s_range) + p->W > max_planes) p->resample.K = 0;
+    }
+    if (p->resample.K > 0) {
+      p->Nt = p->resample.Nt;
+      p->G = p->resample.G;
+    }
+  }
+  const int Nt = p->Nt;
+  const double dlt = p->resample.K > 0 ? p->dl * p->resample.d : p->dl;
   p->logG = 0;
   while ((1 << p->logG) < p->G) ++p->logG;
   p->nT = p->G / p->T;
-  p->dl = p->fov / N;
   p->beta = 2.30 * p->W;
-  const double half = 0.5 * N * p->dl;
+  const double half = 0.5 * Nt * dlt;
   const double r2c = 2.0 * half * half;
   const double s_min = -r2c / (1.0 + std::sqrt(1.0 - r2c));
   const double s_max = 0.0;
@@ -647,13 +678,13 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   // ---- tables: ES transform, twiddles, per-pixel corrections
   std::vector<double> gx, gw;
   gauss_legendre01(kGlNodes, gx, gw);
-  std::vector<double> psi(N);
-  for (int i = 0; i < N; ++i) psi[i] = psi_hat_host((double)(i - N / 2) / p->G, p->W, p->beta, gx, gw);
+  std::vector<double> psi(Nt);
+  for (int i = 0; i < Nt; ++i) psi[i] = psi_hat_host((double)(i - Nt / 2) / p->G, p->W, p->beta, gx, gw);
   double *d_psi, *d_gx, *d_gw;
-  PC_TRY(tmp.alloc((void**)&d_psi, sizeof(double) * (N + 2 * kGlNodes)));
-  d_gx = d_psi + N;
+  PC_TRY(tmp.alloc((void**)&d_psi, sizeof(double) * (Nt + 2 * kGlNodes)));
+  d_gx = d_psi + Nt;
   d_gw = d_gx + kGlNodes;
-  PC_CUDA(cudaMemcpyAsync(d_psi, psi.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st));
+  PC_CUDA(cudaMemcpyAsync(d_psi, psi.data(), sizeof(double) * Nt, cudaMemcpyHostToDevice, st));
   // node factors of the w-kernel correction: W z_q and w_q phi(z_q)
   std::vector<double> wz(kGlNodes), wphi(kGlNodes);
   for (int q = 0; q < kGlNodes; ++q) {
@@ -662,16 +693,27 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   }
   PC_CUDA(cudaMemcpyAsync(d_gx, wz.data(), sizeof(double) * kGlNodes, cudaMemcpyHostToDevice, st));
   PC_CUDA(cudaMemcpyAsync(d_gw, wphi.data(), sizeof(double) * kGlNodes, cudaMemcpyHostToDevice, st));
-  const int64_t NN = (int64_t)N * N;
-  PC_TRY(dev_alloc_t(p, &p->pix_tab, NN));
+  const int64_t NN = (int64_t)N * N, NNt = (int64_t)Nt * Nt;
+  PC_TRY(dev_alloc_t(p, &p->pix_tab, NNt));
   {
-    PixGeom pg{p->dl, p->w0, p->dw, p->s_c, p->beta, N, p->W, p->wstack};
-    k_pix_tab<<<ceil_div(NN, 256), 256, 0, st>>>(pg, d_psi, d_gx, d_gw, kGlNodes, p->pix_tab);
+    PixGeom pg{dlt, p->w0, p->dw, p->s_c, p->beta, Nt, p->W, p->wstack};
+    k_pix_tab<<<ceil_div(NNt, 256), 256, 0, st>>>(pg, d_psi, d_gx, d_gw, kGlNodes, p->pix_tab);
     PC_LAUNCH_CHECK();
   }
   PC_TRY(dev_alloc_t(p, &p->atom_tab, NN));
   k_atom_tab<<<ceil_div(NN, 256), 256, 0, st>>>(N, p->dl, p->atom_tab);
   PC_LAUNCH_CHECK();
+  if (p->resample.K > 0) {
+    resample_widths(p->resample, N, &p->up.width, &p->down.width);
+    const int gu = ceil_div(N, 8), gd = ceil_div(Nt, 8);
+    PC_TRY(dev_alloc_t(p, &p->up.first, (size_t)gu));
+    PC_TRY(dev_alloc_t(p, &p->up.w, (size_t)gu * p->up.width * 8));
+    PC_TRY(dev_alloc_t(p, &p->down.first, (size_t)gd));
+    PC_TRY(dev_alloc_t(p, &p->down.w, (size_t)gd * p->down.width * 8));
+    PC_TRY(dev_alloc_t(p, &p->small_img, (size_t)NNt));
+    PC_TRY(dev_alloc_t(p, &p->small_tmp, (size_t)Nt * N));
+    PC_TRY(fill_band_tables(p->resample, N, &p->up, &p->down, st));
+  }
   std::vector<float2> tw(p->G);
   for (int k = 0; k < p->G; ++k) {
     double a = 2.0 * M_PI * k / p->G;
@@ -711,10 +753,10 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   // larger grids only when those passes can be chosen: forced, or timed by
   // the autotuner; the one-CTA passes use the compact buffer xc instead)
   if (!fft_big_size(p->G) || p->fft_warp == 0 || p->want_tune) {
-    PC_TRY(dev_alloc_t(p, &p->fft1, (size_t)p->P * N * p->G));
+    PC_TRY(dev_alloc_t(p, &p->fft1, (size_t)p->P * Nt * p->G));
     // columns b of the transposed pass-1 output whose grid rows never hold a
     // visibility stay zero for every certificate: clear them once here
-    PC_CUDA(cudaMemsetAsync(p->fft1, 0, sizeof(float2) * (size_t)p->P * N * p->G, st));
+    PC_CUDA(cudaMemsetAsync(p->fft1, 0, sizeof(float2) * (size_t)p->P * Nt * p->G, st));
   }
   PC_TRY(dev_alloc_t(p, &p->resid, (size_t)std::max<int64_t>(M, 1)));
   PC_TRY(dev_alloc_t(p, &p->mu, (size_t)NN));
@@ -754,7 +796,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   const int nblk = ceil_div(nkeys, RS_ITEMS);
   PC_TRY(tmp.alloc((void**)&hist, sizeof(unsigned) * 256 * (size_t)nblk));
   PC_TRY(tmp.alloc((void**)&off, sizeof(int) * ((size_t)nbins + 1)));
-  BinGeom bg{p->dl, p->w0, p->dw, p->s_c, p->G, p->T, p->nT, p->W, p->P, p->Pw, nbins};
+  BinGeom bg{dlt, p->w0, p->dw, p->s_c, p->dl, p->G, p->T, p->nT, p->W, p->P, p->Pw, nbins};
   k_vis_prep<<<ceil_div(M, 256), 256, 0, st>>>(uvw, M, bg, p->vis_fx, k0, v0);
   PC_LAUNCH_CHECK();
 
@@ -882,7 +924,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
     if (fft_big_size(p->G)) {
       // the one-CTA passes' compact rows, allocated here (never inside a captured solve)
       const size_t nb = (size_t)ceil_div(std::max(p->n_active_rows, 1), 4);
-      PC_TRY(p->xc.ensure(sizeof(float2) * (size_t)p->P * nb * N * 4));
+      PC_TRY(p->xc.ensure(sizeof(float2) * (size_t)p->P * nb * Nt * 4));
       PC_TRY(make_xc_tensor_map(p));
     }
   }
@@ -1049,7 +1091,7 @@ extern "C" int pc_plan(const double* uvw_dev, int64_t M, int32_t N, double fov_r
 extern "C" int pc_plan_info(pc_plan_t p, int32_t* grid_side, int32_t* tile, int32_t* n_planes,
                             int64_t* n_slots, int32_t* kernel_width, double* dw) {
   if (!p) return fail(PC_ERR_INVALID_ARG, "pc_plan_info: NULL plan");
-  if (grid_side) *grid_side = p->G;
+  if (grid_side) *grid_side = p->G_image;
   if (tile) *tile = p->T;
   if (n_planes) *n_planes = p->P;
   if (n_slots) *n_slots = p->n_slots;

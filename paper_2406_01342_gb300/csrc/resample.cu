@@ -1,0 +1,238 @@
+// Transforms at the resolution of the visibilities.
+//
+// An image is usually sampled finer than its visibilities resolve: a source's
+// response turns |u| dl times per pixel, 0.08 to 0.28 in the configurations, where
+// the image could hold 0.5. The w-plane transforms then run on a smaller image of
+// the same field (side Nt = G / 2, pixels d times wider, so the grid's side G is
+// 2 to 4 times smaller and its cells stay as wide as they were), and the sum of
+// the planes, corrected and real, is interpolated to the N x N pixels:
+//
+//   img[i][j] = sum_{k, l < K} g(x_i - k) g(x_j - l) small[k][l],  x_i = (i - N/2) / d + Nt/2,
+//   g(x) = sinc(x) I0(beta sqrt(1 - (2x/K)^2)) / I0(beta),  beta = pi K (1/2 - nu),
+//
+// the Kaiser-windowed sinc, for a band |frequency| <= nu cycles per small pixel
+// (nu from max |u|, |v| and the slope of the w-term over the field). With beta >=
+// 14.9, the rule below, it is within 1.5e-7 (rms 5e-8) of e^{2 pi i f x} over the
+// band: a twentieth of the operators' own error. The forward operator runs the
+// transpose.
+//
+// Both directions are one kernel run twice: a banded matrix applied along the
+// rows, the result stored transposed. Each thread holds one column and eight
+// consecutive output rows, whose bands overlap, so an input value is loaded once
+// for eight products; the weights come from a table of eight per input row
+// (zeros outside a band), broadcast from shared memory. What bounds it: those
+// shared-memory reads, three for eight products.
+#include <cmath>
+
+#include "pc_internal.cuh"
+
+namespace pc {
+namespace {
+
+constexpr int RS_COLS = 128;   // columns (threads) per CTA
+constexpr int RS_ROWS = 32;    // output rows per CTA: four groups of eight
+
+__device__ double bessel_i0(double x) {   // power series, 1e-16 relative in about 2 x terms
+  const double q = 0.25 * x * x;
+  double term = 1.0, sum = 1.0;
+  for (int k = 1; k < 200 && term > 1e-17 * sum; ++k) {
+    term *= q / ((double)k * k);
+    sum += term;
+  }
+  return sum;
+}
+
+struct Taps {
+  double d, beta, i0_beta;
+  int N, Nt, K;
+};
+
+__host__ __device__ inline double tap_x(const Taps& t, int i) { return (i - t.N / 2) / t.d + t.Nt / 2; }
+__host__ __device__ inline int tap_first(const Taps& t, int i) { return (int)floor(tap_x(t, i)) - t.K / 2 + 1; }
+
+__device__ double tap_weight(const Taps& t, int i, int k) {
+  const double x = tap_x(t, i) - k, z = 2.0 * x / t.K;
+  if (!(fabs(z) < 1.0)) return 0.0;
+  const double s = fabs(x) < 1e-9 ? 1.0 : sinpi(x) / (M_PI * x);
+  return s * bessel_i0(t.beta * sqrt(1.0 - z * z)) / t.i0_beta;
+}
+
+// Band tables: group g of eight output rows starts at input row first[g] and
+// holds `width` rows of eight weights. Up: output rows are the N pixels; down:
+// the Nt small ones (the transpose).
+__global__ void k_band_table(Taps t, int up, int groups, int width, int* __restrict__ first,
+                             float* __restrict__ w) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= groups * width * 8) return;
+  const int r = e & 7, in = (e >> 3) % width, g = (e >> 3) / width;
+  const int out = 8 * g + r;
+  int f;
+  if (up) {
+    f = tap_first(t, 8 * g);
+  } else {
+    // first pixel whose taps reach row 8 g: tap_first(i) + K > 8 g
+    f = (int)ceil((8 * g - t.K / 2 - t.Nt / 2) * t.d) + t.N / 2 - 2;
+    f = max(f, 0);
+    while (f < t.N && tap_first(t, f) + t.K <= 8 * g) ++f;
+  }
+  if (r == 0 && in == 0) first[g] = f;
+  double v = 0.0;
+  if (up) {
+    const int k = f + in;
+    if (out < t.N && k >= 0 && k < t.Nt) {
+      const int k0 = tap_first(t, out);
+      if (k >= k0 && k < k0 + t.K) v = tap_weight(t, out, k);
+    }
+  } else {
+    const int i = f + in;
+    if (out < t.Nt && i < t.N) {
+      const int k0 = tap_first(t, i);
+      if (out >= k0 && out < k0 + t.K) v = tap_weight(t, i, out);
+    }
+  }
+  w[e] = (float)v;
+}
+
+// out[c][o] = scale * sum_t w[o][t] in[first + t][c]: in has n_in rows of n_cols,
+// out n_cols rows of n_out (transposed). The last application of the adjoint
+// also takes the maxima (maxbits, as the FFT epilogue).
+__global__ void __launch_bounds__(RS_COLS)
+k_band_apply(const float* __restrict__ in, int n_in, int n_cols, const int* __restrict__ first,
+             const float* __restrict__ w, int width, float* __restrict__ out, int n_out, float scale,
+             unsigned* __restrict__ maxbits) {
+  extern __shared__ float4 rs_w[];                         // 4 groups x width x 8 weights
+  __shared__ float tile[RS_ROWS][RS_COLS + 1];
+  const int tid = threadIdx.x;
+  const int c0 = blockIdx.x * RS_COLS, o0 = blockIdx.y * RS_ROWS;
+  const int c = min(c0 + tid, n_cols - 1);
+  const int groups = (n_out + 7) / 8, g0 = o0 / 8, gn = min(RS_ROWS / 8, groups - g0);
+  const float4* src = reinterpret_cast<const float4*>(w) + (size_t)g0 * width * 2;
+  for (int e = tid; e < gn * width * 2; e += RS_COLS) rs_w[e] = src[e];
+  __syncthreads();
+  for (int g = 0; g < gn; ++g) {
+    const int f = first[g0 + g];
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float4* wg = rs_w + (size_t)g * width * 2;
+#pragma unroll 4
+    for (int t = 0; t < width; ++t) {
+      const float v = in[(size_t)min(max(f + t, 0), n_in - 1) * n_cols + c];
+      const float4 a = wg[2 * t], b = wg[2 * t + 1];
+      acc[0] = fmaf(a.x, v, acc[0]);
+      acc[1] = fmaf(a.y, v, acc[1]);
+      acc[2] = fmaf(a.z, v, acc[2]);
+      acc[3] = fmaf(a.w, v, acc[3]);
+      acc[4] = fmaf(b.x, v, acc[4]);
+      acc[5] = fmaf(b.y, v, acc[5]);
+      acc[6] = fmaf(b.z, v, acc[6]);
+      acc[7] = fmaf(b.w, v, acc[7]);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) tile[8 * g + r][tid] = acc[r] * scale;
+  }
+  __syncthreads();
+  // 32 consecutive outputs of one column per warp
+  const int lane = tid & 31, warp = tid >> 5, o = o0 + lane;
+  float amax = 0.f;
+  unsigned skey = 0;   // order-preserving key of the signed maximum (0 below every number)
+  if (o < n_out) {
+    for (int q = warp; q < RS_COLS && c0 + q < n_cols; q += RS_COLS / 32) {
+      const float m = tile[lane][q];
+      out[(size_t)(c0 + q) * n_out + o] = m;
+      amax = fmaxf(amax, fabsf(m));
+      if (m != m) amax = __int_as_float(0x7fc00000);
+      skey = max(skey, float_order_key(m));
+    }
+  }
+  if (!maxbits) return;
+  unsigned bits = __float_as_uint(amax);
+  for (int off = 16; off; off >>= 1) {
+    bits = max(bits, __shfl_xor_sync(0xffffffffu, bits, off));
+    skey = max(skey, __shfl_xor_sync(0xffffffffu, skey, off));
+  }
+  if (lane == 0) {
+    atomicMax(maxbits, bits);
+    atomicMax(maxbits + 1, skey);
+  }
+}
+
+int apply(const float* in, int n_in, int n_cols, const BandTable& t, float* out, int n_out, float scale,
+          unsigned* maxbits, cudaStream_t st) {
+  const size_t smem = (size_t)(RS_ROWS / 8) * t.width * 8 * sizeof(float);
+  static bool attr = false;
+  if (!attr) {
+    PC_CUDA(cudaFuncSetAttribute(k_band_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    attr = true;
+  }
+  k_band_apply<<<dim3(ceil_div(n_cols, RS_COLS), ceil_div(n_out, RS_ROWS)), RS_COLS, smem, st>>>(
+      in, n_in, n_cols, t.first, t.w, t.width, out, n_out, scale, maxbits);
+  PC_LAUNCH_CHECK();
+  return PC_OK;
+}
+
+}  // namespace
+
+// The smallest grid of side 512 or more whose image of side G / 2 still samples
+// the visibilities: with K taps (16 .. 40) past the field's edge the pixels are d
+// = N / (G / 2 - K) wide, and K must reach beta = 14.9. turns: the most that a
+// visibility turns per image pixel, w-term included. Only grids of side 2048 and
+// more are replaced: at 1024 the passes take 28 us of a 512 x 512 certificate's
+// 220, which the interpolation and a wider field's further w-planes would eat.
+Resample choose_resample(int N, int G, double turns) {
+  Resample r;
+  r.Nt = N;
+  r.G = G;
+  if (G < 2048) return r;
+  for (int g = 512; g < G; g *= 2)
+    for (int K = 16; K <= 40; K += 8) {
+      const double d = (double)N / (g / 2 - K), nu = turns * d, beta = M_PI * K * (0.5 - nu);
+      if (d < 1.0 || beta < 14.9) continue;
+      r.K = K;
+      r.Nt = g / 2;
+      r.G = g;
+      r.d = d;
+      r.beta = beta;
+      return r;
+    }
+  return r;
+}
+
+// Rows of the two tables: the widest band of eight output rows.
+void resample_widths(const Resample& r, int N, int* up, int* down) {
+  const Taps t{r.d, r.beta, 1.0, N, r.Nt, r.K};
+  int wu = 0, wd = 0;
+  for (int i = 0; i < N; i += 8) wu = std::max(wu, tap_first(t, std::min(i + 7, N - 1)) + r.K - tap_first(t, i));
+  // an input pixel i meets rows [first, first + K): those of eight rows span at
+  // most (K + 7) d + 2 pixels
+  wd = (int)std::ceil((r.K + 7) * r.d) + 2;
+  *up = wu + 1;   // the device may round a pixel that falls on a small one the other way
+  *down = wd;
+}
+
+int fill_band_tables(const Resample& r, int N, BandTable* up, BandTable* down, cudaStream_t st) {
+  double i0 = 1.0, term = 1.0;
+  for (int k = 1; k < 200; ++k) {
+    term *= 0.25 * r.beta * r.beta / ((double)k * k);
+    i0 += term;
+  }
+  const Taps t{r.d, r.beta, i0, N, r.Nt, r.K};
+  const int gu = ceil_div(N, 8), gd = ceil_div(r.Nt, 8);
+  k_band_table<<<ceil_div((int64_t)gu * up->width * 8, 256), 256, 0, st>>>(t, 1, gu, up->width, up->first, up->w);
+  k_band_table<<<ceil_div((int64_t)gd * down->width * 8, 256), 256, 0, st>>>(t, 0, gd, down->width, down->first,
+                                                                             down->w);
+  PC_LAUNCH_CHECK();
+  return PC_OK;
+}
+
+// img (N x N) = scale * interpolation of the plan's small image
+int launch_upsample(pc_plan_s* p, float* img, float scale, unsigned* maxbits, cudaStream_t st) {
+  PC_TRY(apply(p->small_img, p->Nt, p->Nt, p->up, p->small_tmp, p->N, 1.0f, nullptr, st));
+  return apply(p->small_tmp, p->Nt, p->N, p->up, img, p->N, scale, maxbits, st);
+}
+
+// the plan's small image = the transpose applied to img
+int launch_downsample(pc_plan_s* p, const float* img, cudaStream_t st) {
+  PC_TRY(apply(img, p->N, p->N, p->down, p->small_tmp, p->Nt, 1.0f, nullptr, st));
+  return apply(p->small_tmp, p->N, p->Nt, p->down, p->small_img, p->Nt, 1.0f, nullptr, st);
+}
+
+}  // namespace pc

@@ -426,7 +426,8 @@ int run_operator_apgd(pc_plan_s* p, const float2* V, const float* dirty, const i
   const int gb = std::min(ceil_div(n, 256), 1024);
   int flag = 0;
   // the image rows that hold the atoms: the one-CTA FFT passes of the
-  // operator pairs transform only those on the image side
+  // operator pairs transform only those on the image side (transforms on a
+  // smaller image take all their rows: a band of 16 to 40 around each atom's)
   struct Restrict {
     pc_plan_s* p;
     ~Restrict() {
@@ -435,7 +436,7 @@ int run_operator_apgd(pc_plan_s* p, const float2* V, const float* dirty, const i
       p->img_row_bits = nullptr;
     }
   } restrict_guard{p};
-  if (fft_big_size(p->G)) {
+  if (fft_big_size(p->G) && p->resample.K == 0) {
     {
       ProfScope ps(PROF_APGD_OP, st);
       ps.kernels = 1;
