@@ -282,9 +282,6 @@ bool grid_win_mode(const pc_plan_s* p);   // the plan grids (and degrids) over p
 // degrid_win.cu: degridding interpolation over plane windows, one thread per
 // slot (y added to)
 int launch_degrid_win(pc_plan_s* p, float2* y, cudaStream_t st);
-// plan.cu: window gridding CTAs for at most `cap` slots each
-int split_wsubs(pc_plan_s* p, int cap, cudaStream_t st);
-int split_dwsubs(pc_plan_s* p, int cap, cudaStream_t st);
 int launch_fft_rows(pc_plan_s* p, cudaStream_t st);
 int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
                              cudaStream_t st);

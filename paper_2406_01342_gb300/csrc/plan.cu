@@ -60,16 +60,47 @@ static void gauss_legendre01(int n, std::vector<double>& x, std::vector<double>&
 }
 
 // Fourier transform of the ES kernel in cell units at frequency t (cycles per cell):
-//   psi(t) = int_{-W/2}^{W/2} phi(2y/W) e^{-j 2 pi y t} dy = W int_0^1 phi(z) cos(pi W z t) dz.
-static double psi_hat_host(double t, int W, double beta, const std::vector<double>& gx,
-                           const std::vector<double>& gw) {
+//   psi(t) = int_{-W/2}^{W/2} phi(2y/W) e^{-j 2 pi y t} dy = W int_0^1 phi(z) cos(pi W z t) dz
+// = W sum_q wphi[q] cos(pi wz[q] t) by quadrature (wz = W z_q, wphi = w_q phi(z_q)).
+static double psi_hat_host(double t, int W, const std::vector<double>& wz, const std::vector<double>& wphi) {
   double s = 0.0;
-  for (size_t q = 0; q < gx.size(); ++q) {
-    double z = gx[q];
-    double phi = std::exp(beta * (std::sqrt(std::max(0.0, 1.0 - z * z)) - 1.0));
-    s += gw[q] * phi * std::cos(M_PI * W * z * t);
-  }
+  for (size_t q = 0; q < wz.size(); ++q) s += wphi[q] * std::cos(M_PI * wz[q] * t);
   return W * s;
+}
+
+// psi(k / G) for k <= n, the cosines by their three-term recurrence (n <= G / 4:
+// its rounding stays below 1e-10).
+static void psi_hat_grid(int n, int G, int W, const std::vector<double>& wz, const std::vector<double>& wphi,
+                         std::vector<double>& out) {
+  out.assign((size_t)n + 1, 0.0);
+  for (size_t q = 0; q < wz.size(); ++q) {
+    const double c1 = std::cos(M_PI * wz[q] / G);
+    double c = 1.0, cm = c1;
+    for (int k = 0; k <= n; ++k) {
+      out[(size_t)k] += wphi[q] * c;
+      const double cn = 2.0 * c1 * c - cm;
+      cm = c;
+      c = cn;
+    }
+  }
+  for (double& v : out) v *= W;
+}
+
+// Chebyshev coefficients in y = 2 (t / T)^2 - 1 of 1 / psi(t), |t| <= T = 1/4: the
+// w-kernel's correction as a polynomial (psi is entire and even: 16 terms leave
+// 1e-12).
+constexpr int kPsiTerms = 16;
+static void psi_poly(double T, int W, const std::vector<double>& wz, const std::vector<double>& wphi, double* c) {
+  double f[kPsiTerms];
+  for (int i = 0; i < kPsiTerms; ++i) {
+    const double y = std::cos(M_PI * (i + 0.5) / kPsiTerms);
+    f[i] = 1.0 / psi_hat_host(T * std::sqrt(0.5 * (y + 1.0)), W, wz, wphi);
+  }
+  for (int k = 0; k < kPsiTerms; ++k) {
+    double v = 0.0;
+    for (int i = 0; i < kPsiTerms; ++i) v += f[i] * std::cos(M_PI * k * (i + 0.5) / kPsiTerms);
+    c[k] = v * (k ? 2.0 : 1.0) / kPsiTerms;
+  }
 }
 
 // ------------------------------------------------------------------ device kernels
@@ -197,47 +228,59 @@ __global__ void k_rs_hist(const unsigned* __restrict__ keys, int64_t n, int shif
   hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
 }
 
-// Exclusive scan of L unsigned values by one block of 1024 threads.
-__global__ void k_scan_single(unsigned* __restrict__ a, int64_t L) {
-  __shared__ unsigned warp_tot[32];
-  int64_t chunk = (L + blockDim.x - 1) / blockDim.x;
-  int64_t lo = threadIdx.x * chunk, hi = lo + chunk < L ? lo + chunk : L;
-  unsigned s = 0;
-  for (int64_t i = lo; i < hi; ++i) s += a[i];
-  // block exclusive scan of s
-  unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned incl = s;
-  for (int off = 1; off < 32; off <<= 1) {
-    unsigned t = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += t;
-  }
-  if (lane == 31) warp_tot[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    unsigned t = warp_tot[lane];
-    unsigned ti = t;
+// Exclusive scan over the blocks of every digit's counts (block d: digit d), in
+// place, and the digits' totals. The scatter adds up the totals itself. One block
+// over all digits read 256 nblk entries through one SM: 2.5M entries and most of a
+// 10M-visibility plan's 26 ms.
+__global__ void __launch_bounds__(256) k_rs_scan(unsigned* __restrict__ hist, int nblk, unsigned* __restrict__ total) {
+  __shared__ unsigned warp_tot[8];
+  unsigned* row = hist + (int64_t)blockIdx.x * nblk;
+  const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned run = 0;
+  for (int base = 0; base < nblk; base += 256) {
+    const int i = base + (int)threadIdx.x;
+    const unsigned v = i < nblk ? row[i] : 0u;
+    unsigned incl = v;
     for (int off = 1; off < 32; off <<= 1) {
-      unsigned u = __shfl_up_sync(0xffffffffu, ti, off);
-      if (lane >= off) ti += u;
+      const unsigned t = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= (unsigned)off) incl += t;
     }
-    warp_tot[lane] = ti - t;
+    if (lane == 31) warp_tot[wid] = incl;
+    __syncthreads();
+    unsigned before = 0, all = 0;
+    for (unsigned w = 0; w < 8; ++w) {
+      before += w < wid ? warp_tot[w] : 0u;
+      all += warp_tot[w];
+    }
+    if (i < nblk) row[i] = run + before + incl - v;
+    run += all;
+    __syncthreads();
   }
-  __syncthreads();
-  unsigned run = warp_tot[wid] + incl - s;
-  for (int64_t i = lo; i < hi; ++i) {
-    unsigned v = a[i];
-    a[i] = run;
-    run += v;
-  }
+  if (threadIdx.x == 0) total[blockIdx.x] = run;
 }
 
 __global__ void k_rs_scatter(const unsigned* __restrict__ kin, const unsigned* __restrict__ vin,
                              unsigned* __restrict__ kout, unsigned* __restrict__ vout, int64_t n,
-                             int shift, const unsigned* __restrict__ hist, int nblk) {
+                             int shift, const unsigned* __restrict__ hist, int nblk,
+                             const unsigned* __restrict__ total) {
   __shared__ unsigned s_base[256];
+  __shared__ unsigned s_tot[RS_THREADS / 32];
   __shared__ unsigned s_w[RS_THREADS / 32][256];
   int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  s_base[tid] = hist[(int64_t)tid * nblk + blockIdx.x];
+  {
+    // first position of digit tid: the totals of the digits before it
+    const unsigned t = total[tid];
+    unsigned incl = t;
+    for (int off = 1; off < 32; off <<= 1) {
+      const unsigned o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    if (lane == 31) s_tot[warp] = incl;
+    __syncthreads();
+    unsigned before = 0;
+    for (int w = 0; w < warp; ++w) before += s_tot[w];
+    s_base[tid] = before + incl - t + hist[(int64_t)tid * nblk + blockIdx.x];
+  }
   int64_t base = (int64_t)blockIdx.x * RS_ITEMS;
   unsigned lt_mask = (1u << lane) - 1u;
   for (int r = 0; r < RS_ROUNDS; ++r) {
@@ -269,14 +312,19 @@ __global__ void k_rs_scatter(const unsigned* __restrict__ kin, const unsigned* _
   }
 }
 
-// off[b] = first sorted position with key >= b, for b in [0, nbins]; keys <= nbins.
+// off[b] = first sorted position whose bin is >= b, for b in [0, nbins]; the keys
+// of unused slots (bin nbins) come last. A search per bin: one thread per key,
+// filling the empty bins before it, left thousands to single threads.
 __global__ void k_bin_offsets(const unsigned* __restrict__ keys, int64_t n, unsigned nbins,
                               int* __restrict__ off) {
-  int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (j > n) return;
-  long long kcur = j < n ? (long long)(keys[j] >> kBinSubBits) : (long long)nbins;
-  long long kprev = j == 0 ? -1 : (long long)(keys[j - 1] >> kBinSubBits);
-  for (long long b = kprev + 1; b <= kcur && b <= (long long)nbins; ++b) off[b] = (int)j;
+  const unsigned b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b > nbins) return;
+  int64_t lo = 0, hi = n;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if ((keys[mid] >> kBinSubBits) < b) lo = mid + 1; else hi = mid;
+  }
+  off[b] = (int)lo;
 }
 
 // Slot records in sorted order.
@@ -316,47 +364,81 @@ struct PixGeom {
   bool wstack;
 };
 
-// Per-pixel epilogue coefficients: {Re, Im} of e^{j 2 pi w0 s} / (n psi(i') psi(j') psi_w(t))
-// and t = dw (s - s_c) as a double-float (hi, lo).
-__global__ void k_pix_tab(PixGeom g, const double* __restrict__ psi_uv,
-                          const double* __restrict__ glx, const double* __restrict__ glw,
-                          int nq, float4* __restrict__ out) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t NN = (int64_t)g.N * g.N;
-  if (p >= NN) return;
-  int i = (int)(p / g.N), j = (int)(p % g.N);
-  double l = (i - g.N / 2) * g.dl, m = (j - g.N / 2) * g.dl;
+// Per-pixel tables are even in the pixel's offsets i' = i - N/2, j' = j - N/2: a
+// thread per quadrant pixel evaluates its FP64 square root and divisions (a slow
+// pipe on this GPU) once and writes the up to four pixels (+-i', +-j').
+template <class T, class F>
+__device__ __forceinline__ void write_quadrant(T* __restrict__ out, int N, int a, int b, F value) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ip = q & 2 ? -a : a, jp = q & 1 ? -b : b;
+    if ((q & 2 && a == 0) || (q & 1 && b == 0) || ip >= N / 2 || jp >= N / 2) continue;
+    out[(size_t)(ip + N / 2) * N + (jp + N / 2)] = value(ip, jp);
+  }
+}
+
+// Epilogue coefficients: {Re, Im} of e^{j 2 pi w0 s} / (n psi(i') psi(j') psi_w(t))
+// and t = dw (s - s_c) as a double-float (hi, lo). rpsi: 1 / psi(k / G), k <= N/2;
+// poly: 1 / psi_w(t) (psi_poly).
+__global__ void k_pix_tab(PixGeom g, const double* __restrict__ rpsi, const double* __restrict__ poly,
+                          float4* __restrict__ out) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
+  if (b > g.N / 2) return;
+  double l = a * g.dl, m = b * g.dl;
   double r2 = l * l + m * m;
   double n = sqrt(1.0 - r2);
   double s = -r2 / (1.0 + n);        // n - 1 without cancellation
-  double t = 0.0, psiw = 1.0;
+  double t = 0.0, rw = 1.0;
   if (g.wstack) {
-    // psi_w(t) = W sum_q w_q phi(z_q) cos(pi W z_q t): glx holds W z_q and glw
-    // w_q phi(z_q) (node-only factors, from the host); |W z_q t| <= W/4, where an
-    // FP32 cosine is accurate to ~1e-7
     t = g.dw * (s - g.s_c);
-    double acc = 0.0;
-    for (int q = 0; q < nq; ++q) acc += glw[q] * (double)cospif((float)(glx[q] * t));
-    psiw = g.W * acc;
+    const double y = 32.0 * t * t - 1.0;            // 2 (t / T)^2 - 1, T = 1/4
+    double b1 = 0.0, b2 = 0.0;
+#pragma unroll
+    for (int k = kPsiTerms - 1; k >= 1; --k) {
+      const double v = 2.0 * y * b1 - b2 + poly[k];
+      b2 = b1;
+      b1 = v;
+    }
+    rw = y * b1 - b2 + poly[0];
   }
   double ct = g.w0 * s;
   ct -= rint(ct);                    // exact reduction to [-1/2, 1/2] turns in FP64
   float snf, csf;                    // then an FP32 sine / cosine (~1e-7): FP64 ones are slow here
   sincospif(2.0f * (float)ct, &snf, &csf);
-  const double sn = snf, cs = csf;
-  double d = 1.0 / (n * psi_uv[i] * psi_uv[j] * psiw);
-  float t_hi = (float)t;
-  float t_lo = (float)(t - (double)t_hi);
-  out[p] = make_float4((float)(cs * d), (float)(sn * d), t_hi, t_lo);
+  const double d = rpsi[a] * rpsi[b] * rw / n;
+  const float t_hi = (float)t;
+  const float4 v = make_float4((float)((double)csf * d), (float)((double)snf * d), t_hi, (float)(t - (double)t_hi));
+  write_quadrant(out, g.N, a, b, [&](int, int) { return v; });
 }
 
-// Per-pixel unit-weight atoms, evaluated once per plan: their s = n - 1 and
-// 1 / n take FP64 square roots and divisions, a slow pipe on this GPU, which
-// the solver's per-iteration bookkeeping then only gathers.
+// Per-pixel unit-weight atoms, evaluated once per plan; the solver's
+// per-iteration bookkeeping then only gathers them.
 __global__ void k_atom_tab(int N, double dl, float4* __restrict__ out) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= (int64_t)N * N) return;
-  out[p] = make_atom((int)p, 1.f, false, N, dl);
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
+  if (b > N / 2) return;
+  // pixel (-a, -b) exists for every a, b <= N/2
+  const float4 at = make_atom((N / 2 - a) * N + (N / 2 - b), 1.f, false, N, dl);
+  write_quadrant(out, N, a, b, [&](int ip, int jp) {
+    return make_float4(__int_as_float((int)(((unsigned)ip << 16) | ((unsigned)jp & 0xffffu))), at.y, at.z, at.w);
+  });
+}
+
+// FFT twiddle tables: tw[k] = e^{+2 pi i k / G}; tw2 [k1 < G/32][l < 32] of the
+// one-warp FFT (G = 512, 1024); tw_in [k1 < 16][l < 32] and tw_big [k1 < G/512][n'
+// < 512] of the one-CTA FFT (G >= 2048). Null tables are left out.
+__global__ void k_twiddles(int G, float2* __restrict__ tw, float2* __restrict__ tw2, float2* __restrict__ tw_in,
+                           float2* __restrict__ tw_big) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= G) return;
+  auto root = [&](int e) {
+    double sn, cs;
+    sincospi(2.0 * (e % G) / G, &sn, &cs);
+    return make_float2((float)cs, (float)sn);
+  };
+  tw[k] = root(k);
+  if (tw2) tw2[k] = root((k >> 5) * (k & 31));                       // G entries
+  if (tw_in && k < 512) tw_in[k] = root((k >> 5) * (k & 31) * (G / 512));
+  if (tw_big) tw_big[k] = root((k >> 9) * (k & 511));
 }
 
 // The stream plan construction runs on: plan buffers come from the library's
@@ -374,6 +456,46 @@ template <class T>
 static int dev_alloc_t(pc_plan_s* p, T** ptr, size_t count) {
   return dev_alloc(p, reinterpret_cast<void**>(ptr), count * sizeof(T));
 }
+
+// Host arrays on their way to or from the device, in recycled pinned memory, so
+// that a copy neither waits for the stream nor for the host array's lifetime (a
+// copy from pageable memory waits for the stream first: thirteen of them kept host
+// and device taking turns). Chunks of powers of two, so that plans of other sizes
+// reuse them; released after the stream has been waited for.
+struct Staging {
+  std::vector<void*> chunks;
+  char* at = nullptr;
+  size_t left = 0;
+  cudaStream_t st = nullptr;
+  ~Staging() {
+    if (!chunks.empty()) cudaStreamSynchronize(st);
+    for (void* q : chunks) pinned_put(q);
+  }
+  void* block(size_t bytes) {
+    bytes = (bytes + 15) / 16 * 16;
+    if (bytes > left) {
+      size_t chunk = 256 * 1024;
+      while (chunk < bytes) chunk *= 2;
+      void* q = pinned_get(chunk);
+      if (!q) return nullptr;
+      chunks.push_back(q);
+      at = static_cast<char*>(q);
+      left = chunk;
+    }
+    void* q = at;
+    at += bytes;
+    left -= bytes;
+    return q;
+  }
+  int upload(void* dst, const void* src, size_t bytes) {
+    if (bytes == 0) return PC_OK;
+    void* q = block(bytes);
+    if (!q) return fail(PC_ERR_OOM, "plan: %zu bytes of pinned memory", bytes);
+    std::memcpy(q, src, bytes);
+    PC_CUDA(cudaMemcpyAsync(dst, q, bytes, cudaMemcpyHostToDevice, st));
+    return PC_OK;
+  }
+};
 
 // Temporary device buffers of plan construction, freed on every exit path.
 struct TmpBufs {
@@ -394,7 +516,7 @@ struct TmpBufs {
 // Window CTAs: a tile whose slots exceed `cap` is split into equal parts
 // (each part takes its share of every plane window of the tile); heaviest
 // CTAs first, so the last wave holds the light ones.
-static int split_win_parts(pc_plan_s* p, int cap, int4* dst, int* n_out, cudaStream_t st) {
+static int split_win_parts(pc_plan_s* p, int cap, int4* dst, int* n_out, Staging& up) {
   cap = std::max(cap, 64);
   std::vector<int4> subs;
   for (const int2& t : p->win_tiles) {
@@ -404,28 +526,25 @@ static int split_win_parts(pc_plan_s* p, int cap, int4* dst, int* n_out, cudaStr
   std::stable_sort(subs.begin(), subs.end(), [](const int4& a, const int4& b) { return a.w > b.w; });
   if ((int64_t)subs.size() > p->wsub_cap) return fail(PC_ERR_CAPACITY, "plan: %zu window CTAs", subs.size());
   *n_out = (int)subs.size();
-  if (!subs.empty())
-    PC_CUDA(cudaMemcpyAsync(dst, subs.data(), sizeof(int4) * subs.size(), cudaMemcpyHostToDevice, st));
-  PC_CUDA(cudaStreamSynchronize(st));   // the host vector goes out of scope
-  return PC_OK;
+  return up.upload(dst, subs.data(), sizeof(int4) * subs.size());
 }
 
 // The window gridding's CTAs (each part adds its tile to the grid).
-int split_wsubs(pc_plan_s* p, int cap, cudaStream_t st) {
-  PC_TRY(split_win_parts(p, cap, p->wsubs, &p->n_wsub, st));
+static int split_wsubs(pc_plan_s* p, int cap, Staging& up) {
+  PC_TRY(split_win_parts(p, cap, p->wsubs, &p->n_wsub, up));
   p->win_cap = std::max(cap, 64);
   return PC_OK;
 }
 
 // The window degridding's CTAs (each part reads its tile's planes; no part
 // writes the grid, so the split only costs plane loads).
-int split_dwsubs(pc_plan_s* p, int cap, cudaStream_t st) {
-  PC_TRY(split_win_parts(p, cap, p->dwsubs, &p->n_dwsub, st));
+static int split_dwsubs(pc_plan_s* p, int cap, Staging& up) {
+  PC_TRY(split_win_parts(p, cap, p->dwsubs, &p->n_dwsub, up));
   p->dwin_cap = std::max(cap, 64);
   return PC_OK;
 }
 
-static int split_subs(pc_plan_s* p, int piece, cudaStream_t st) {
+static int split_subs(pc_plan_s* p, int piece, Staging& up) {
   std::vector<int4> subs;
   for (const int4& r : p->sub_ranges) {
     const int len = r.w - r.z;
@@ -436,10 +555,7 @@ static int split_subs(pc_plan_s* p, int piece, cudaStream_t st) {
   if ((int)subs.size() > p->sub_cap) return fail(PC_ERR_CAPACITY, "plan: %zu sub-problems", subs.size());
   p->n_sub = (int)subs.size();
   p->grid_piece = piece;
-  if (!subs.empty())
-    PC_CUDA(cudaMemcpyAsync(p->subs, subs.data(), sizeof(int4) * subs.size(), cudaMemcpyHostToDevice, st));
-  PC_CUDA(cudaStreamSynchronize(st));   // the host vector goes out of scope
-  return PC_OK;
+  return up.upload(p->subs, subs.data(), sizeof(int4) * subs.size());
 }
 
 __global__ void k_fill_ones(float2* __restrict__ h, int64_t M) {
@@ -478,6 +594,8 @@ static int time_us(cudaStream_t st, int reps, F f, double* out) {
 // fastest of each.
 static int autotune(pc_plan_s* p, cudaStream_t st) {
   if (p->M <= 0 || p->n_sub == 0) return PC_OK;
+  Staging up;
+  up.st = st;
   k_fill_ones<<<(int)std::min<int64_t>(4096, (p->M + 255) / 256), 256, 0, st>>>(p->resid, p->M);
   PC_LAUNCH_CHECK();
   const int user_mode = p->grid_mode;
@@ -493,7 +611,7 @@ static int autotune(pc_plan_s* p, cudaStream_t st) {
                                         : std::vector<int>{256, 512, 1024, 2048, 4096};
     for (int piece : pieces) {
       p->grid_mode = mode;
-      PC_TRY(win ? split_wsubs(p, piece, st) : split_subs(p, piece, st));
+      PC_TRY(win ? split_wsubs(p, piece, up) : split_subs(p, piece, up));
       double us = 0.0;
       PC_TRY(time_us(st, 3, [&] { return launch_grid(p, p->resid, st); }, &us));
       if (us < best) {
@@ -504,7 +622,7 @@ static int autotune(pc_plan_s* p, cudaStream_t st) {
     }
   }
   p->grid_mode = best_mode;
-  PC_TRY(grid_win_mode(p) ? split_wsubs(p, best_piece, st) : split_subs(p, best_piece, st));
+  PC_TRY(grid_win_mode(p) ? split_wsubs(p, best_piece, up) : split_subs(p, best_piece, up));
   p->tune_grid_us = best;
   PC_TRY(launch_grid(p, p->resid, st));         // a gridded plane set for the FFT timing
   // first pass: the one-warp register FFT (where G allows it) against the
@@ -563,7 +681,7 @@ static int autotune(pc_plan_s* p, cudaStream_t st) {
     double best_dw = 1e300;
     int best_cap = p->dwin_cap;
     for (int cap : {2048, 4096, 8192, 16384}) {
-      PC_TRY(split_dwsubs(p, cap, st));
+      PC_TRY(split_dwsubs(p, cap, up));
       double us = 0.0;
       PC_TRY(time_us(st, 3, [&] { return launch_degrid_win(p, p->resid, st); }, &us));
       if (us < best_dw) {
@@ -571,7 +689,7 @@ static int autotune(pc_plan_s* p, cudaStream_t st) {
         best_cap = cap;
       }
     }
-    PC_TRY(split_dwsubs(p, best_cap, st));
+    PC_TRY(split_dwsubs(p, best_cap, up));
     p->tune_degrid_us = best_dw;
   }
   p->tuned = true;
@@ -586,6 +704,8 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   g_build_stream = st;
   TmpBufs tmp;
   tmp.st = st;
+  Staging up;
+  up.st = st;
 
   // ---- w range, largest |u|, |v| and finiteness
   double uv_max = 0.0;
@@ -594,19 +714,16 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
     int* dbad;
     PC_TRY(tmp.alloc((void**)&dmm, 3 * sizeof(unsigned long long) + sizeof(int) * 2));
     dbad = reinterpret_cast<int*>(dmm + 3);
-    unsigned long long init[3] = {~0ull, 0ull, 0ull};
-    int zero[2] = {0, 0};
-    PC_CUDA(cudaMemcpyAsync(dmm, init, sizeof(init), cudaMemcpyHostToDevice, st));
-    PC_CUDA(cudaMemcpyAsync(dbad, zero, sizeof(zero), cudaMemcpyHostToDevice, st));
+    PC_CUDA(cudaMemsetAsync(dmm, 0xff, sizeof(unsigned long long), st));
+    PC_CUDA(cudaMemsetAsync(dmm + 1, 0, 2 * sizeof(unsigned long long) + 2 * sizeof(int), st));
     int blocks = (int)std::min<int64_t>(4096, (M + 255) / 256);
     k_uvw_scan<<<blocks, 256, 0, st>>>(uvw, M, dmm, dmm + 1, dmm + 2, dbad);
     PC_LAUNCH_CHECK();
-    unsigned long long hmm[3];
-    int hbad[2];
-    PC_CUDA(cudaMemcpyAsync(hmm, dmm, sizeof(hmm), cudaMemcpyDeviceToHost, st));
-    PC_CUDA(cudaMemcpyAsync(hbad, dbad, sizeof(hbad), cudaMemcpyDeviceToHost, st));
+    struct { unsigned long long mm[3]; int bad[2]; } got;
+    PC_CUDA(cudaMemcpyAsync(&got, dmm, sizeof(got), cudaMemcpyDeviceToHost, st));
     PC_CUDA(cudaStreamSynchronize(st));
-    if (hbad[0]) return fail(PC_ERR_INVALID_ARG, "plan: uvw contains NaN or Inf");
+    const unsigned long long* hmm = got.mm;
+    if (got.bad[0]) return fail(PC_ERR_INVALID_ARG, "plan: uvw contains NaN or Inf");
     auto unmap = [](unsigned long long o) {
       unsigned long long b = (o & 0x8000000000000000ull) ? (o & 0x7fffffffffffffffull) : ~o;
       double d;
@@ -678,30 +795,30 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   // ---- tables: ES transform, twiddles, per-pixel corrections
   std::vector<double> gx, gw;
   gauss_legendre01(kGlNodes, gx, gw);
-  std::vector<double> psi(Nt);
-  for (int i = 0; i < Nt; ++i) psi[i] = psi_hat_host((double)(i - Nt / 2) / p->G, p->W, p->beta, gx, gw);
-  double *d_psi, *d_gx, *d_gw;
-  PC_TRY(tmp.alloc((void**)&d_psi, sizeof(double) * (Nt + 2 * kGlNodes)));
-  d_gx = d_psi + Nt;
-  d_gw = d_gx + kGlNodes;
-  PC_CUDA(cudaMemcpyAsync(d_psi, psi.data(), sizeof(double) * Nt, cudaMemcpyHostToDevice, st));
-  // node factors of the w-kernel correction: W z_q and w_q phi(z_q)
+  // node factors of the quadrature: W z_q and w_q phi(z_q)
   std::vector<double> wz(kGlNodes), wphi(kGlNodes);
   for (int q = 0; q < kGlNodes; ++q) {
     wz[q] = p->W * gx[q];
     wphi[q] = gw[q] * std::exp(p->beta * (std::sqrt(std::max(0.0, 1.0 - gx[q] * gx[q])) - 1.0));
   }
-  PC_CUDA(cudaMemcpyAsync(d_gx, wz.data(), sizeof(double) * kGlNodes, cudaMemcpyHostToDevice, st));
-  PC_CUDA(cudaMemcpyAsync(d_gw, wphi.data(), sizeof(double) * kGlNodes, cudaMemcpyHostToDevice, st));
+  std::vector<double> rpsi;
+  psi_hat_grid(Nt / 2, p->G, p->W, wz, wphi, rpsi);
+  for (double& v : rpsi) v = 1.0 / v;
+  rpsi.resize(rpsi.size() + kPsiTerms);
+  double* poly = rpsi.data() + Nt / 2 + 1;
+  psi_poly(0.25, p->W, wz, wphi, poly);
+  double* d_psi;
+  PC_TRY(tmp.alloc((void**)&d_psi, sizeof(double) * rpsi.size()));
+  PC_TRY(up.upload(d_psi, rpsi.data(), sizeof(double) * rpsi.size()));
   const int64_t NN = (int64_t)N * N, NNt = (int64_t)Nt * Nt;
   PC_TRY(dev_alloc_t(p, &p->pix_tab, NNt));
   {
     PixGeom pg{dlt, p->w0, p->dw, p->s_c, p->beta, Nt, p->W, p->wstack};
-    k_pix_tab<<<ceil_div(NNt, 256), 256, 0, st>>>(pg, d_psi, d_gx, d_gw, kGlNodes, p->pix_tab);
+    k_pix_tab<<<dim3(ceil_div(Nt / 2 + 1, 128), Nt / 2 + 1), 128, 0, st>>>(pg, d_psi, d_psi + Nt / 2 + 1, p->pix_tab);
     PC_LAUNCH_CHECK();
   }
   PC_TRY(dev_alloc_t(p, &p->atom_tab, NN));
-  k_atom_tab<<<ceil_div(NN, 256), 256, 0, st>>>(N, p->dl, p->atom_tab);
+  k_atom_tab<<<dim3(ceil_div(N / 2 + 1, 128), N / 2 + 1), 128, 0, st>>>(N, p->dl, p->atom_tab);
   PC_LAUNCH_CHECK();
   if (p->resample.K > 0) {
     resample_widths(p->resample, N, &p->up.width, &p->down.width);
@@ -714,49 +831,27 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
     PC_TRY(dev_alloc_t(p, &p->small_tmp, (size_t)Nt * N));
     PC_TRY(fill_band_tables(p->resample, N, &p->up, &p->down, st));
   }
-  std::vector<float2> tw(p->G);
-  for (int k = 0; k < p->G; ++k) {
-    double a = 2.0 * M_PI * k / p->G;
-    tw[k] = make_float2((float)std::cos(a), (float)std::sin(a));
-  }
   PC_TRY(dev_alloc_t(p, &p->twiddle, p->G));
-  PC_CUDA(cudaMemcpyAsync(p->twiddle, tw.data(), sizeof(float2) * p->G, cudaMemcpyHostToDevice, st));
-  if (p->G == 512 || p->G == 1024) {
-    const int L = p->G / 32;
-    std::vector<float2> t2((size_t)32 * L);
-    for (int k1 = 0; k1 < L; ++k1)
-      for (int l = 0; l < 32; ++l) t2[(size_t)k1 * 32 + l] = tw[(size_t)(k1 * l) % p->G];
-    PC_TRY(dev_alloc_t(p, &p->tw2, t2.size()));
-    PC_CUDA(cudaMemcpyAsync(p->tw2, t2.data(), sizeof(float2) * t2.size(), cudaMemcpyHostToDevice, st));
-  }
-
+  if (p->G == 512 || p->G == 1024) PC_TRY(dev_alloc_t(p, &p->tw2, p->G));
   if (fft_big_size(p->G)) {
-    // the 512-point one-warp FFT inside the one-CTA transform: e^{+2 pi i l k1 / 512}
-    std::vector<float2> t2(16 * 32);
-    const int step = p->G / 512;
-    for (int k1 = 0; k1 < 16; ++k1)
-      for (int l = 0; l < 32; ++l) t2[(size_t)k1 * 32 + l] = tw[(size_t)(k1 * l * step) % p->G];
-    PC_TRY(dev_alloc_t(p, &p->tw_in, t2.size()));
-    PC_CUDA(cudaMemcpyAsync(p->tw_in, t2.data(), sizeof(float2) * t2.size(), cudaMemcpyHostToDevice, st));
-    // its first step's twiddles by (k1, n'): e^{+2 pi i n' k1 / G}, n' < 512
-    std::vector<float2> ta((size_t)p->G);
-    for (int k1 = 0; k1 < p->G / 512; ++k1)
-      for (int n = 0; n < 512; ++n) ta[(size_t)k1 * 512 + n] = tw[((size_t)n * k1) % p->G];
-    PC_TRY(dev_alloc_t(p, &p->tw_big, ta.size()));
-    PC_CUDA(cudaMemcpyAsync(p->tw_big, ta.data(), sizeof(float2) * ta.size(), cudaMemcpyHostToDevice, st));
+    PC_TRY(dev_alloc_t(p, &p->tw_in, 512));
+    PC_TRY(dev_alloc_t(p, &p->tw_big, p->G));
   }
+  k_twiddles<<<ceil_div(p->G, 128), 128, 0, st>>>(p->G, p->twiddle, p->tw2, p->tw_in, p->tw_big);
+  PC_LAUNCH_CHECK();
 
   // ---- workspaces
   PC_TRY(dev_alloc_t(p, &p->grid, (size_t)p->P * p->G * p->G));
-  PC_CUDA(cudaMemsetAsync(p->grid, 0, sizeof(float2) * (size_t)p->P * p->G * p->G, st));
+  // only the Stockham passes read cells that no visibility reaches (whole rows of
+  // the grid, whole columns of their transposed output): those stay zero from here
+  const bool whole_rows = !(p->G == 512 || p->G == 1024 || fft_big_size(p->G)) || p->fft_warp == 0 || p->want_tune;
+  if (whole_rows) PC_CUDA(cudaMemsetAsync(p->grid, 0, sizeof(float2) * (size_t)p->P * p->G * p->G, st));
   // the Stockham passes' transposed pass-1 output (every G up to 1024; for
   // larger grids only when those passes can be chosen: forced, or timed by
   // the autotuner; the one-CTA passes use the compact buffer xc instead)
   if (!fft_big_size(p->G) || p->fft_warp == 0 || p->want_tune) {
     PC_TRY(dev_alloc_t(p, &p->fft1, (size_t)p->P * Nt * p->G));
-    // columns b of the transposed pass-1 output whose grid rows never hold a
-    // visibility stay zero for every certificate: clear them once here
-    PC_CUDA(cudaMemsetAsync(p->fft1, 0, sizeof(float2) * (size_t)p->P * Nt * p->G, st));
+    if (whole_rows) PC_CUDA(cudaMemsetAsync(p->fft1, 0, sizeof(float2) * (size_t)p->P * Nt * p->G, st));
   }
   PC_TRY(dev_alloc_t(p, &p->resid, (size_t)std::max<int64_t>(M, 1)));
   PC_TRY(dev_alloc_t(p, &p->mu, (size_t)NN));
@@ -794,7 +889,8 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   PC_TRY(tmp.alloc((void**)&v0, sizeof(unsigned) * nkeys));
   PC_TRY(tmp.alloc((void**)&v1, sizeof(unsigned) * nkeys));
   const int nblk = ceil_div(nkeys, RS_ITEMS);
-  PC_TRY(tmp.alloc((void**)&hist, sizeof(unsigned) * 256 * (size_t)nblk));
+  PC_TRY(tmp.alloc((void**)&hist, sizeof(unsigned) * 256 * ((size_t)nblk + 1)));
+  unsigned* const total = hist + 256 * (size_t)nblk;
   PC_TRY(tmp.alloc((void**)&off, sizeof(int) * ((size_t)nbins + 1)));
   BinGeom bg{dlt, p->w0, p->dw, p->s_c, p->dl, p->G, p->T, p->nT, p->W, p->P, p->Pw, nbins};
   k_vis_prep<<<ceil_div(M, 256), 256, 0, st>>>(uvw, M, bg, p->vis_fx, k0, v0);
@@ -807,17 +903,18 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   for (int shift = 0; shift < nbits; shift += 8) {
     k_rs_hist<<<nblk, RS_THREADS, 0, st>>>(kin, nkeys, shift, hist, nblk);
     PC_LAUNCH_CHECK();
-    k_scan_single<<<1, 1024, 0, st>>>(hist, 256 * (int64_t)nblk);
+    k_rs_scan<<<256, 256, 0, st>>>(hist, nblk, total);
     PC_LAUNCH_CHECK();
-    k_rs_scatter<<<nblk, RS_THREADS, 0, st>>>(kin, vin, kout, vout, nkeys, shift, hist, nblk);
+    k_rs_scatter<<<nblk, RS_THREADS, 0, st>>>(kin, vin, kout, vout, nkeys, shift, hist, nblk, total);
     PC_LAUNCH_CHECK();
     std::swap(kin, kout);
     std::swap(vin, vout);
   }
-  k_bin_offsets<<<ceil_div(nkeys + 1, 256), 256, 0, st>>>(kin, nkeys, nbins, off);
+  k_bin_offsets<<<ceil_div((int64_t)nbins + 1, 256), 256, 0, st>>>(kin, nkeys, nbins, off);
   PC_LAUNCH_CHECK();
-  std::vector<int> hoff((size_t)nbins + 1);
-  PC_CUDA(cudaMemcpyAsync(hoff.data(), off, sizeof(int) * hoff.size(), cudaMemcpyDeviceToHost, st));
+  const int* hoff = static_cast<const int*>(up.block(sizeof(int) * ((size_t)nbins + 1)));
+  if (!hoff) return fail(PC_ERR_OOM, "plan: pinned memory for %u bins", nbins);
+  PC_CUDA(cudaMemcpyAsync(const_cast<int*>(hoff), off, sizeof(int) * ((size_t)nbins + 1), cudaMemcpyDeviceToHost, st));
   PC_CUDA(cudaStreamSynchronize(st));
   p->n_slots = hoff[nbins];
 
@@ -873,7 +970,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   // room for the finest split the autotuner may try (pieces of 64 slots)
   p->sub_cap = (int)(total_slots / 64 + (int64_t)ranges.size() + 1);
   PC_TRY(dev_alloc_t(p, &p->subs, (size_t)p->sub_cap));
-  PC_TRY(split_subs(p, piece, st));
+  PC_TRY(split_subs(p, piece, up));
   // window gridding: the bin offsets on the device, the tiles that hold slots,
   // and the CTA list. Measured (2048^2 / 2M and 4096^2 / 10M): splitting a
   // tile costs more than it balances once the tiles alone give eight CTAs per
@@ -888,11 +985,11 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   }
   p->wsub_cap = p->n_slots / 64 + (int64_t)p->win_tiles.size() + 1;
   PC_TRY(dev_alloc_t(p, &p->wsubs, (size_t)p->wsub_cap));
-  PC_TRY(split_wsubs(p, (int64_t)p->win_tiles.size() >= 8ll * n_sm ? 65536 : 4096, st));
+  PC_TRY(split_wsubs(p, (int64_t)p->win_tiles.size() >= 8ll * n_sm ? 65536 : 4096, up));
   PC_TRY(dev_alloc_t(p, &p->dwsubs, (size_t)p->wsub_cap));
   // window degridding: parts of at most 8192 slots (measured best or within
   // 2 % of the best cap on 2048^2 / 2M and 4096^2 / 10M; the tuner times it)
-  PC_TRY(split_dwsubs(p, 8192, st));
+  PC_TRY(split_dwsubs(p, 8192, up));
   // grid rows that any visibility can reach: the rows of tile rows with a sub-problem
   {
     std::vector<char> row_on(p->nT, 0);
@@ -903,14 +1000,12 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
         for (int b = 0; b < p->T; ++b) rows.push_back(tv * p->T + b);
     p->n_active_rows = (int)rows.size();
     PC_TRY(dev_alloc_t(p, &p->active_rows, std::max<size_t>(rows.size(), 1)));
-    if (!rows.empty())
-      PC_CUDA(cudaMemcpyAsync(p->active_rows, rows.data(), sizeof(int) * rows.size(),
-                              cudaMemcpyHostToDevice, st));
+    PC_TRY(up.upload(p->active_rows, rows.data(), sizeof(int) * rows.size()));
     // compact position of every grid row, and the column groups that can hold data
     std::vector<int> pos(p->G, -1);
     for (size_t c = 0; c < rows.size(); ++c) pos[rows[c]] = (int)c;
     PC_TRY(dev_alloc_t(p, &p->row_pos, (size_t)p->G));
-    PC_CUDA(cudaMemcpyAsync(p->row_pos, pos.data(), sizeof(int) * p->G, cudaMemcpyHostToDevice, st));
+    PC_TRY(up.upload(p->row_pos, pos.data(), sizeof(int) * p->G));
     std::vector<uint32_t> colw((size_t)std::max(1, p->G / 1024), 0u);
     for (const int4& s : ranges) {
       const int g = s.x % p->nT;                  // a tile column is one 32-column group
@@ -919,8 +1014,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
     p->n_active_col_groups = 0;
     for (uint32_t word : colw) p->n_active_col_groups += __builtin_popcount(word);
     PC_TRY(dev_alloc_t(p, &p->col_bits, colw.size()));
-    PC_CUDA(cudaMemcpyAsync(p->col_bits, colw.data(), sizeof(uint32_t) * colw.size(), cudaMemcpyHostToDevice,
-                            st));
+    PC_TRY(up.upload(p->col_bits, colw.data(), sizeof(uint32_t) * colw.size()));
     if (fft_big_size(p->G)) {
       // the one-CTA passes' compact rows, allocated here (never inside a captured solve)
       const size_t nb = (size_t)ceil_div(std::max(p->n_active_rows, 1), 4);
