@@ -13,10 +13,10 @@
 // Ritz values approach the top eigenvalue from below and converge faster than
 // linearly, so the 1 % margin of L covers the remaining error many times.
 //
-// GB300 mapping: one thread-block cluster, as few CTAs as let each CTA keep
-// its rows of G in shared memory (1 CTA up to n ~ 220, 16 for n ~ 900). CTA r
-// owns a contiguous block of rows of G and of every vector. Each iteration does
-// one GEMV: the CTAs publish their slice of the proximal point z in shared
+// GB300 mapping: one CTA up to 224 atoms (k_apgd_cta), a thread-block cluster of
+// 8 or 16 beyond (k_apgd_full), and k_apgd where the full vectors do not fit: a
+// cluster whose CTA r owns a contiguous block of rows of G and of every vector.
+// Each of its iterations does one GEMV: the CTAs publish their slice of the proximal point z in shared
 // memory, a cluster barrier, every CTA gathers the whole z through distributed
 // shared memory, multiplies its rows, publishes its partial sums, a second
 // barrier, and every CTA reduces the partials in the same order (so all take
@@ -97,8 +97,9 @@ struct ApgdArgs {
   int positive;   // 1: x >= 0 (proximal map max(z - lambda/L, 0))
   int rows_per;
   int n_pad;
-  int cache;      // 1: rows of G cached in shared memory
+  int cache;      // rows of G that a CTA keeps in shared memory (k_apgd: 1 for all, 0 for none)
   int vec_ok;     // 1: float4 loads of G rows are aligned
+  int scalar;     // k_apgd_full: a lane takes single columns, not groups of four
 };
 
 // Rows [r0, r0 + nr) of G (leading dimension ldg, n columns) into dst (row
@@ -239,13 +240,13 @@ __device__ void gemv_rows(const Smem& s, const ApgdArgs& a, int r0, int nr, floa
   }
 }
 
-// Block-wide double-float sums of NPART per-thread values, written to part[] by thread 0.
+// Double-float sums of NPART values over the block's first APGD_THREADS threads, written to part[].
 __device__ void block_sums(Df v[NPART], Df* part, Df* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = APGD_THREADS / 32;
   for (int off = 16; off; off >>= 1)
 #pragma unroll
     for (int q = 0; q < NPART; ++q) v[q] = df_add(v[q], df_shfl_xor(v[q], off));
-  if (lane == 0)
+  if (lane == 0 && warp < nw)
 #pragma unroll
     for (int q = 0; q < NPART; ++q) scratch[warp * NPART + q] = v[q];
   __syncthreads();
@@ -452,58 +453,63 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd(const __grid_constant_
   cl.sync();   // no CTA leaves while others may still read its shared memory
 }
 
-// Block-wide FP32 sums of K per-thread values (a fixed butterfly: the same
-// inputs give the same sums in every CTA); every thread receives them.
+// FP32 sums of K values over the block's first APGD_THREADS threads (a fixed
+// butterfly: the same inputs give the same sums in every CTA), for every thread. One
+// barrier: the buffers alternate, and every thread adds the eight warps' sums.
 template <int K>
-__device__ void block_sum_f(float (&v)[K], float* scratch, float* out) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int off = 16; off; off >>= 1)
-#pragma unroll
-    for (int q = 0; q < K; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < K; ++q) scratch[warp * K + q] = v[q];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int q = 0; q < K; ++q) v[q] = lane < nw ? scratch[lane * K + q] : 0.f;
-    for (int off = 4; off; off >>= 1)
+__device__ __forceinline__ void block_sum_f(float (&v)[K], float (*red)[3][8], int& parity) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < APGD_THREADS / 32) {
+    for (int off = 16; off; off >>= 1)
 #pragma unroll
       for (int q = 0; q < K; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
     if (lane == 0)
 #pragma unroll
-      for (int q = 0; q < K; ++q) out[q] = v[q];
+      for (int q = 0; q < K; ++q) red[parity][q][warp] = v[q];
   }
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < K; ++q) v[q] = out[q];
+  for (int q = 0; q < K; ++q) {
+    const float4 f = *reinterpret_cast<const float4*>(&red[parity][q][0]);
+    const float4 h = *reinterpret_cast<const float4*>(&red[parity][q][4]);
+    v[q] = ((f.x + h.x) + (f.z + h.z)) + ((f.y + h.y) + (f.w + h.w));
+  }
+  parity ^= 1;
 }
 
 // ---------------------------------------------------------------------------
 // Full-vector variant (used whenever its vectors fit): every CTA keeps all n
 // entries of x, y, z, Gx, Gy and b, and owns rows [r0, r0 + nr) of G (nr a
-// multiple of 4 except in the last CTA). A matrix-vector product multiplies
-// the own rows by the (local) full vector into a local slice and PUSHES the
-// slice to every CTA of the cluster with one bulk copy each (shared memory to
-// distributed shared memory), whose bytes complete on the receiver's
-// mbarrier; each CTA then waits (bounded) on its own mbarrier until all
-// entries have landed. No cluster barrier and no remote loads sit on the
-// iteration path, only the one-way latency of the copies.
-// The reductions and updates are then done redundantly over all n entries --
-// identical data and order in every CTA, hence identical decisions.
+// multiple of 4 except in the last CTA), as many of them in shared memory as fit;
+// the others are read from L2 each time, 16 loads of 16 bytes in flight a thread.
+// A warp multiplies four rows by the (local) full vector and sends the four sums
+// to every CTA of the cluster, a lane to each, as one asynchronous 16-byte store
+// whose bytes complete on the receiver's mbarrier; every thread then waits
+// (bounded) on its CTA's mbarrier until all entries have landed. No cluster
+// barrier and no remote loads sit on the iteration path, only the one-way
+// latency of the stores. The reductions and updates are then done redundantly
+// over all n entries -- identical data and order in every CTA, hence identical
+// decisions. Every thread keeps to its own entries of the vectors, so that an
+// iteration crosses two block barriers (input vector complete; partial sums
+// complete).
 //
-// Two receive buffers (and two local slices) alternate. A CTA pushes product
-// i + 2 into buffer i mod 2 only after it has received every CTA's product
-// i + 1, which each CTA sends only after it has consumed product i and
-// re-armed that buffer's mbarrier, so a buffer is never overwritten while it
-// is read, bytes never arrive before the phase that counts them is armed, and
-// a local slice is rewritten only after every copy that read it has landed.
+// Two receive buffers alternate. A CTA sends product i + 2 into buffer i mod 2
+// only after it has received every CTA's product i + 1, which each CTA sends only
+// after it has consumed product i, so a buffer is never overwritten while it is
+// read. The mbarrier of a buffer is re-armed for product i + 2 before this CTA
+// sends product i + 1, and no phase can end twice while a thread still waits for
+// its first end: product i + 2 needs this CTA's own rows, which it sends after a
+// barrier of all its threads.
+//
+// What bounds it: up to 800 atoms the latency of exchange, barriers and sums;
+// beyond, the rows that 16 SMs cannot keep, read from L2. Measured against bulk
+// copies of slices with six barriers an iteration, all rows or none in shared
+// memory, us an iteration before and after: 300 atoms 2.30 and 1.46, 500 2.50 and
+// 1.68, 900 5.5 and 3.8, 1300 7.2 and 5.7, 2500 16.8 and 16.0.
 
 constexpr long long APGD_WAIT_CYCLES = 4000000000ll;   // ~2 s at 2 GHz
 
 struct SmemF {
-  float* pub0;    // rows_per each: this CTA's slices of the last two products
-  float* pub1;
   float* rx0;     // n_pad each: the two receive buffers of the products
   float* rx1;
   float* x;       // n_pad each, full vectors
@@ -512,14 +518,12 @@ struct SmemF {
   float* Gy;
   float* z;
   float* bb;
-  float* Gc;      // rows_per x n_pad (optional)
+  float* Gc;      // cache x n_pad
 };
 
 __device__ SmemF carve_full(float* base, const ApgdArgs& a) {
   SmemF s;
   float* p = base;
-  s.pub0 = p; p += a.rows_per;
-  s.pub1 = p; p += a.rows_per;
   s.rx0 = p; p += a.n_pad;
   s.rx1 = p; p += a.n_pad;
   s.x = p; p += a.n_pad;
@@ -568,94 +572,89 @@ struct Exchange {
   __device__ uint32_t bar(int b) const { return b ? bar1 : bar0; }
 };
 
+// Four rows of G by a vector in shared memory: the lane's part. U: steps of the
+// column loop whose loads are issued together.
+template <int U>
+__device__ __forceinline__ void rows_dot(const float* const (&rows)[4], const float* vec, int n, bool vecld,
+                                         float (&acc)[4]) {
+  const int lane = threadIdx.x & 31, n4 = n >> 2;
+  const float4* v4 = reinterpret_cast<const float4*>(vec);
+  if (vecld) {
+#pragma unroll U
+    for (int c = lane; c < n4; c += 32) {
+      const float4 z = v4[c];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 g = reinterpret_cast<const float4*>(rows[q])[c];
+        acc[q] = fmaf(g.x, z.x, acc[q]);
+        acc[q] = fmaf(g.y, z.y, acc[q]);
+        acc[q] = fmaf(g.z, z.z, acc[q]);
+        acc[q] = fmaf(g.w, z.w, acc[q]);
+      }
+    }
+    for (int c = 4 * n4 + lane; c < n; c += 32)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = fmaf(rows[q][c], vec[c], acc[q]);
+  } else {
+#pragma unroll U
+    for (int c = lane; c < n; c += 32)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = fmaf(rows[q][c], vec[c], acc[q]);
+  }
+}
+
 // G vec for all n rows, in every CTA; returns the receive buffer holding it.
-// *ok becomes false (in every thread of the CTA) if the bounded wait expired.
+// *bad is set if the bounded wait expired: read it behind the next barrier. The
+// caller's barriers order the vector's writes before and its next ones after.
 __device__ float* cluster_gemv(const ApgdArgs& a, const SmemF& s, const float* vec, int r0, int nr,
-                               Exchange& ex, bool& ok) {
+                               Exchange& ex, int* bad) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int b = ex.buf;
-  // a one-CTA cluster writes the product straight into its receive buffer: no
-  // bulk copy to itself, no mbarrier round trip
-  const bool solo = ex.CS == 1;
-  float* pub = solo ? (b ? s.rx1 : s.rx0) : (b ? s.pub1 : s.pub0);
-  const bool vecld = a.cache || a.vec_ok;
-  const int n4 = a.n >> 2;
-  const float4* v4 = reinterpret_cast<const float4*>(vec);
-  for (int rb = 4 * warp; rb < nr; rb += 4 * nw) {
+  // rows from L2 first, the cached ones after
+  const int n_groups = (nr + 3) >> 2;
+  for (int gi = n_groups - 1 - warp; gi >= 0; gi -= nw) {
+    const int rb = 4 * gi;
     const float* rows[4];
-    float acc[4];
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (rb < a.cache) {                               // cache: a multiple of 4, or at least nr
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = min(rb + q, nr - 1);
-      rows[q] = a.cache ? s.Gc + (size_t)r * a.n_pad : a.G + (size_t)(r0 + r) * a.ldg;
-      acc[q] = 0.f;
-    }
-    if (vecld) {
-      for (int c = lane; c < n4; c += 32) {
-        const float4 z = v4[c];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 g = reinterpret_cast<const float4*>(rows[q])[c];
-          acc[q] = fmaf(g.x, z.x, acc[q]);
-          acc[q] = fmaf(g.y, z.y, acc[q]);
-          acc[q] = fmaf(g.z, z.z, acc[q]);
-          acc[q] = fmaf(g.w, z.w, acc[q]);
-        }
-      }
-      for (int c = 4 * n4 + lane; c < a.n; c += 32)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = fmaf(rows[q][c], vec[c], acc[q]);
+      for (int q = 0; q < 4; ++q) rows[q] = s.Gc + (size_t)min(rb + q, nr - 1) * a.n_pad;
+      rows_dot<2>(rows, vec, a.n, !a.scalar, acc);
     } else {
-      for (int c = lane; c < a.n; c += 32)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = fmaf(rows[q][c], vec[c], acc[q]);
+      for (int q = 0; q < 4; ++q) rows[q] = a.G + (size_t)(r0 + min(rb + q, nr - 1)) * a.ldg;
+      rows_dot<4>(rows, vec, a.n, a.vec_ok != 0, acc);
     }
     for (int off = 16; off; off >>= 1)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
-    if (lane < 4 && rb + lane < nr) {
-      float v = acc[0];
+    if (lane < ex.CS) {
 #pragma unroll
       for (int q = 1; q < 4; ++q)
-        if (lane == q) v = acc[q];
-      pub[rb + lane] = v;
+        if (rb + q >= nr) acc[q] = 0.f;               // past the last row: fills the vectors' padding
+      asm volatile(
+          "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+              cluster_addr(ex.rx(b) + (uint32_t)(r0 + rb) * 4u, lane)),
+          "r"(__float_as_uint(acc[0])), "r"(__float_as_uint(acc[1])), "r"(__float_as_uint(acc[2])),
+          "r"(__float_as_uint(acc[3])), "r"(cluster_addr(ex.bar(b), lane))
+          : "memory");
     }
   }
-  // the slice (padded to 4 floats) goes to every CTA in one bulk copy each
-  const int nr4 = (nr + 3) & ~3;
-  for (int r = nr + threadIdx.x; r < nr4; r += blockDim.x) pub[r] = 0.f;
-  if (solo) {
-    __syncthreads();
-    ex.buf ^= 1;
-    return pub;
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();
-  if ((int)threadIdx.x < ex.CS && nr4 > 0) {
-    const int d = threadIdx.x;
-    const uint32_t src = (uint32_t)__cvta_generic_to_shared(pub);
-    const uint32_t dst = cluster_addr(ex.rx(b) + (uint32_t)r0 * 4u, d);
-    asm volatile(
-        "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-        "r"(src), "r"((uint32_t)nr4 * 4u), "r"(cluster_addr(ex.bar(b), d))
-        : "memory");
-  }
-  const bool mine = mbar_wait_cluster(ex.bar(b), (ex.phase >> b) & 1u);
-  ok = !__syncthreads_or(!mine);
-  if (ok) {
-    ex.phase ^= 1u << b;
-    ex.buf ^= 1;
-    // re-arm for this buffer's next use (two products from now)
-    if (threadIdx.x == 0) mbar_arm(ex.bar(b), (uint32_t)a.n_pad * 4u);
-  }
+  if (!mbar_wait_cluster(ex.bar(b), (ex.phase >> b) & 1u)) *bad = 1;
+  ex.phase ^= 1u << b;
+  ex.buf ^= 1;
+  // re-arm for this buffer's next use (two products from now)
+  if (threadIdx.x == 0) mbar_arm(ex.bar(b), (uint32_t)a.n_pad * 4u);
   return b ? s.rx1 : s.rx0;
 }
 
-__global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_constant__ ApgdBatch batch) {
+template <int THREADS>   // the first APGD_THREADS hold the vectors, all of them multiply
+__global__ void __launch_bounds__(THREADS, 1) k_apgd_full(const __grid_constant__ ApgdBatch batch) {
   extern __shared__ __align__(16) float apgdf_sm[];
   __shared__ Df scratch[(APGD_THREADS / 32) * NPART];
   __shared__ Df s_part[NPART];
-  __shared__ float s_fscr[(APGD_THREADS / 32) * 3], s_fout[3];
+  __shared__ __align__(16) float s_red[2][3][8];
+  __shared__ int s_bad;
   __shared__ float s_al[LZ_MAX], s_be[LZ_MAX], s_theta;
   __shared__ __align__(8) uint64_t s_rxbar[2];
   cg::cluster_group cl = cg::this_cluster();
@@ -664,8 +663,10 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
   const SmemF s = carve_full(apgdf_sm, a);
   const int r0 = rank * a.rows_per;
   const int nr = max(0, min(a.n, r0 + a.rows_per) - r0);
-  const int n = a.n, tid = threadIdx.x, nt = blockDim.x;
+  const int n = a.n, tid = threadIdx.x, nt = APGD_THREADS;
+  const int e0 = tid < nt ? tid : a.n_pad;    // first own entry of the vectors (none past the first threads)
   bool ok = true;
+  int parity = 0;
 
   Exchange ex;
   ex.rx0 = (uint32_t)__cvta_generic_to_shared(s.rx0);
@@ -676,6 +677,7 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
   ex.buf = 0;
   ex.CS = (int)cl.num_blocks();
   if (tid == 0) {
+    s_bad = 0;
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(ex.bar(b)));
       mbar_arm(ex.bar(b), (uint32_t)a.n_pad * 4u);
@@ -683,9 +685,9 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
 
-  if (a.cache) load_rows_async(s.Gc, a.n_pad, a.G, a.ldg, r0, nr, n, a.vec_ok != 0);
+  load_rows_async(s.Gc, a.n_pad, a.G, a.ldg, r0, min(nr, a.cache), n, a.vec_ok != 0);
   const float v0 = rsqrtf((float)n);        // Lanczos start: all ones / sqrt(n)
-  for (int i = tid; i < a.n_pad; i += nt) {
+  for (int i = e0; i < a.n_pad; i += nt) {
     const bool in = i < n;
     s.bb[i] = in ? a.b[i] : 0.f;
     s.x[i] = in ? a.x[i] : 0.f;
@@ -697,20 +699,23 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
   // ---- Lipschitz constant: Lanczos (alpha = v^T G v, then beta = ||w||)
   float theta = 0.f, theta_prev = 0.f, beta_prev = 0.f;
   int m = 0;
-  for (int j = 0; j < LZ_MAX && ok; ++j) {
-    float* Gv = cluster_gemv(a, s, s.y, r0, nr, ex, ok);       // G v_j
-    if (!ok) break;
+  for (int j = 0; j < LZ_MAX; ++j) {
+    float* Gv = cluster_gemv(a, s, s.y, r0, nr, ex, &s_bad);   // G v_j
     float va[1] = {0.f};
-    for (int i = tid; i < n; i += nt) va[0] = fmaf(s.y[i], Gv[i], va[0]);
-    block_sum_f<1>(va, s_fscr, s_fout);
+    for (int i = e0; i < n; i += nt) va[0] = fmaf(s.y[i], Gv[i], va[0]);
+    block_sum_f<1>(va, s_red, parity);
+    if (s_bad) {
+      ok = false;
+      break;
+    }
     const float alpha = va[0];
     float vb[1] = {0.f};
-    for (int i = tid; i < n; i += nt) {
+    for (int i = e0; i < n; i += nt) {
       const float w = Gv[i] - alpha * s.y[i] - beta_prev * s.z[i];
       Gv[i] = w;
       vb[0] = fmaf(w, w, vb[0]);
     }
-    block_sum_f<1>(vb, s_fscr, s_fout);
+    block_sum_f<1>(vb, s_red, parity);
     const float beta = sqrtf(fmaxf(vb[0], 0.f));
     if (tid == 0) {
       s_al[j] = alpha;
@@ -725,7 +730,7 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
       theta_prev = theta;
     }
     const float inv = 1.f / beta;
-    for (int i = tid; i < n; i += nt) {
+    for (int i = e0; i < n; i += nt) {
       const float vn = Gv[i] * inv;
       s.z[i] = s.y[i];
       s.y[i] = vn;
@@ -735,19 +740,18 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
   }
   const float L = 1.01f * (theta > 0.f ? theta : 1.f);
   const float invL = 1.f / L;
-  const float thr = a.lam * invL;
+  const float thr = __fmul_rn(a.lam, invL);
 
   // ---- initial G x
   if (ok) {
-    const float* Gxr = cluster_gemv(a, s, s.x, r0, nr, ex, ok);
-    if (ok) {
-      for (int i = tid; i < n; i += nt) {
-        const float gx = Gxr[i];
-        s.Gx[i] = gx;
-        s.y[i] = s.x[i];
-        s.Gy[i] = gx;
-      }
-      __syncthreads();
+    const float* Gxr = cluster_gemv(a, s, s.x, r0, nr, ex, &s_bad);
+    __syncthreads();
+    ok = !s_bad;
+    for (int i = e0; i < n; i += nt) {
+      const float gx = Gxr[i];
+      s.Gx[i] = gx;
+      s.y[i] = s.x[i];
+      s.Gy[i] = gx;
     }
   }
 
@@ -755,18 +759,17 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
   float t = 1.f;
   int it = 0;
   for (it = 1; it <= a.max_iter && ok; ++it) {
-    for (int i = tid; i < n; i += nt) {
+    for (int i = e0; i < n; i += nt) {
       const float u = s.y[i] - (s.Gy[i] - s.bb[i]) * invL;
       s.z[i] = (a.positive ? fmaxf(u - thr, 0.f) : copysignf(fmaxf(fabsf(u) - thr, 0.f), u));
     }
     __syncthreads();
-    const float* Gz = cluster_gemv(a, s, s.z, r0, nr, ex, ok);
-    if (!ok) break;
+    const float* Gz = cluster_gemv(a, s, s.z, r0, nr, ex, &s_bad);
     // F(z) - F(x) = sum_i (z_i - x_i) ((Gz_i + Gx_i) / 2 - b_i) + lambda (|z_i| - |x_i|)
     // (G symmetric): every term vanishes as z -> x, so an FP32 sum resolves the
     // sign of the difference where F itself (~1e7) would need ~50 bits
     float v[3] = {0.f, 0.f, 0.f};
-    for (int i = tid; i < n; i += nt) {
+    for (int i = e0; i < n; i += nt) {
       const float zr = s.z[i], xr = s.x[i];
       const float dF = fmaf(zr - xr, 0.5f * (Gz[i] + s.Gx[i]) - s.bb[i], a.lam * (fabsf(zr) - fabsf(xr)));
       v[0] += dF;
@@ -774,13 +777,17 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
       v[1] = fmaf(d, d, v[1]);
       v[2] = fmaf(zr, zr, v[2]);
     }
-    block_sum_f<3>(v, s_fscr, s_fout);
+    const float t1 = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
+    const float c1 = t / t1, c2 = (t - 1.f) / t1;
+    block_sum_f<3>(v, s_red, parity);
+    if (s_bad) {
+      ok = false;
+      break;
+    }
     const float step = sqrtf(v[1]);
     const float nz = sqrtf(v[2]);
-    const float t1 = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
     const bool accept = v[0] <= 0.f;
-    const float c1 = t / t1, c2 = (t - 1.f) / t1;
-    for (int i = tid; i < n; i += nt) {
+    for (int i = e0; i < n; i += nt) {
       const float xo = s.x[i], Gxo = s.Gx[i];
       const float xn = accept ? s.z[i] : xo;
       const float Gxn = accept ? Gz[i] : Gxo;
@@ -790,7 +797,6 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
       s.Gx[i] = Gxn;
     }
     t = t1;
-    __syncthreads();
     if (step <= a.eps * nz) break;
   }
   if (it > a.max_iter) it = a.max_iter;
@@ -798,7 +804,7 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
   Df Fx = {0.f, 0.f};
   if (ok) {
     Df v[NPART] = {};
-    for (int i = tid; i < n; i += nt) {
+    for (int i = e0; i < n; i += nt) {
       v[0] = df_add(v[0], df_prod(s.x[i], s.Gx[i]));
       v[1] = df_add(v[1], df_prod(s.bb[i], s.x[i]));
       v[2] = df_add(v[2], Df{fabsf(s.x[i]), 0.f});
@@ -806,8 +812,9 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
     block_sums(v, s_part, scratch);
     Fx = df_add(df_add(df_scale(s_part[0], 0.5f), df_neg(s_part[1])), df_scale(s_part[2], a.lam));
   }
+  __syncthreads();
   if (ok) {
-    for (int r = tid; r < nr; r += nt) a.x[r0 + r] = s.x[r0 + r];
+    for (int r = tid; r < nr; r += blockDim.x) a.x[r0 + r] = s.x[r0 + r];
     if (rank == 0 && tid == 0) {
       if (a.out_iters) *a.out_iters = it;
       if (a.out_L) *a.out_L = (double)L;
@@ -827,236 +834,146 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_full(const __grid_cons
 }
 
 // ---------------------------------------------------------------------------
-// One-warp variant for small supports (n <= 64, the later Frank-Wolfe
-// iterations): the same Lanczos step size, monotone FISTA, stop rule and
-// reported objective as k_apgd_full, with G in shared memory, lane l owning
-// rows l and l + 32 of every vector, warp-shuffle reductions and no block or
-// cluster barrier in the loop: an iteration is a few hundred instructions.
-constexpr int WARP_NMAX = 64;
+// One-CTA variant for supports of up to CTA_NMAX atoms: the same Lanczos step
+// size, monotone FISTA, stop rule and reported objective, with two threads per
+// row of G and of every vector. Thread h of a row's two holds the row's columns
+// 4 c + 2 h and 4 c + 2 h + 1 in registers (the last NS of its columns in shared
+// memory where the block's threads leave too few registers) and sums each of the
+// two series in the order of c; a product reads only the broadcast vector. An
+// iteration is a serial chain of two block barriers (input vector complete;
+// partial sums complete), the product and the sums, so everything else is kept
+// off it: one further warp evaluates the momentum's coefficients during the
+// product and the stop test during the next proximal step, which a stop discards.
+// Measured against a thread per row with G in shared memory (and one warp for
+// the whole problem up to 64 atoms), us an iteration before and after: 40 atoms
+// 0.66 and 0.50, 120 1.09 and 0.59, 160 1.31 and 1.03, 224 1.83 and 1.28.
+//
+// Order of the sums: a warp holds 16 rows, every second of 32 consecutive ones
+// (SMALL: every fourth of all 64, rows r and r + 32 first), so that the sums over
+// a warp and then over the warps of a group add as a butterfly over 32 rows (64)
+// does; groups of 32 follow in turn.
+constexpr int WARP_NMAX = 64;    // one tree over all rows
+constexpr int CTA_NMAX = 224;
 
-__device__ __forceinline__ float warp_sum(float v) {
-  for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  return v;
-}
-__device__ __forceinline__ Df warp_df_sum(Df v) {
-  for (int off = 16; off; off >>= 1) v = df_add(v, df_shfl_xor(v, off));
-  return v;
+__device__ __forceinline__ float pair_butterfly(float t, bool from_first) {
+  if (from_first) t += __shfl_xor_sync(0xffffffffu, t, 16);
+  t += __shfl_xor_sync(0xffffffffu, t, 8);
+  t += __shfl_xor_sync(0xffffffffu, t, 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  return t;
 }
 
-__global__ void __launch_bounds__(32) k_apgd_warp(const __grid_constant__ ApgdBatch batch) {
-  __shared__ __align__(16) float vs[WARP_NMAX];
+// sum over rows of a b (SMALL: a fused multiply-add per pair of rows r, r + 32)
+template <bool SMALL>
+__device__ __forceinline__ float pair_product_sum(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  if (!SMALL) return pair_butterfly(p, true);
+  return pair_butterfly(fmaf(a, b, __shfl_xor_sync(0xffffffffu, p, 16)), false);
+}
+
+// block-wide total of the warps' partial sums red[0..)
+template <int GROUPS>
+__device__ __forceinline__ float pair_total(const float* red) {
+  const float4* p = reinterpret_cast<const float4*>(red);
+  if (GROUPS == 0) {                                // SMALL: four warps, one tree
+    const float4 f = p[0];
+    return (f.x + f.z) + (f.y + f.w);
+  }
+  float t = 0.f;
+#pragma unroll
+  for (int g = 0; g < GROUPS; g += 2) {             // zeros past the last group
+    const float4 f = p[g >> 1];
+    t += f.x + f.y;
+    t += f.z + f.w;
+  }
+  return t;
+}
+
+template <int NC, int NS>   // columns per thread (n <= 2 NC), the last NS of them in shared memory
+__global__ void __launch_bounds__(4 * NC + 32, 1) k_apgd_cta(const __grid_constant__ ApgdBatch batch) {
+  constexpr bool SMALL = 2 * NC <= WARP_NMAX;
+  constexpr int GROUPS = SMALL ? 0 : (2 * NC + 31) / 32;
+  constexpr int NR = NC - NS, LDV = NC + 4;         // LDV: the halves of vs in different banks
+  extern __shared__ __align__(16) float4 apgdc_sm[];   // NS / 4 x threads
+  __shared__ __align__(16) float vs[2 * LDV];       // the broadcast input: entry i at [i % 4 / 2][i / 4 * 2 + i % 2]
+  __shared__ __align__(16) float s_red[2][3][16];   // [buffer][value][warp]
+  __shared__ float2 s_mom;                          // momentum coefficients of the iteration
+  __shared__ int s_stop;
+  __shared__ Df s_dred[16 * 3];
   __shared__ float s_al[LZ_MAX], s_be[LZ_MAX], s_theta;
   const ApgdArgs& a = batch.job[blockIdx.x];
-  const int n = a.n, lane = threadIdx.x;
-  const int i0 = lane, i1 = lane + 32;
-  const bool v0ok = i0 < n, v1ok = i1 < n;
-  // the lane's two rows of G live in registers (zero beyond n): every load in
-  // flight at once, and a product reads only the broadcast input vector
-  float g0[WARP_NMAX], g1[WARP_NMAX];
+  const int n = a.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int threads = blockDim.x - 32;              // the last warp holds no rows
+  const int groups = threads >> 6, h = lane & 1;
+  const bool rows_warp = tid < threads;
+  const int row = SMALL ? warp + 4 * (lane >> 1) : 32 * (warp >> 1) + (warp & 1) + 2 * (lane >> 1);
+  const int slot = rows_warp ? tid : 0;             // of apgdc_sm: the last warp has none of its own
+  const bool own = rows_warp && row < n, put = own && h == 0;
+  float* vrow = vs + ((row & 2) ? LDV : 0) + (row >> 2) * 2 + (row & 1);
+  float g[NR];
+  {
+    const float* src = a.G + (size_t)(own ? row : 0) * a.ldg;
+    auto at = [&](int e) {                          // this thread's e-th column
+      const int c = 4 * (e >> 1) + 2 * h + (e & 1);
+      return own && c < n ? src[c] : 0.f;
+    };
 #pragma unroll
-  for (int j = 0; j < WARP_NMAX; ++j) {
-    g0[j] = (v0ok && j < n) ? a.G[(size_t)i0 * a.ldg + j] : 0.f;
-    g1[j] = (v1ok && j < n) ? a.G[(size_t)i1 * a.ldg + j] : 0.f;
+    for (int e = 0; e < NR; ++e) g[e] = at(e);
+    if (NS && rows_warp)
+#pragma unroll
+      for (int e = 0; e < NS; e += 4)
+        apgdc_sm[e / 4 * threads + tid] = make_float4(at(NR + e), at(NR + e + 1), at(NR + e + 2), at(NR + e + 3));
   }
-  float bb0 = v0ok ? a.b[i0] : 0.f, bb1 = v1ok ? a.b[i1] : 0.f;
-  float x0 = v0ok ? a.x[i0] : 0.f, x1 = v1ok ? a.x[i1] : 0.f;
-  // G v for the lane's two rows (v broadcast through shared memory, 16-byte
-  // reads; four partial sums per row for independent FMA chains)
-  auto gemv = [&](float v0, float v1, float& g0o, float& g1o) {
-    vs[i0] = v0;
-    vs[i1] = v1;
-    __syncwarp();
-    float p0[4] = {0.f, 0.f, 0.f, 0.f}, p1[4] = {0.f, 0.f, 0.f, 0.f};
-    const float4* v4 = reinterpret_cast<const float4*>(vs);
+  auto product = [&]() {
+    const float4* v4 = reinterpret_cast<const float4*>(vs + h * LDV);
+    float a0 = 0.f, a1 = 0.f;
 #pragma unroll
-    for (int j4 = 0; j4 < WARP_NMAX / 4; ++j4) {
-      const float4 z = v4[j4];
-      p0[0] = fmaf(g0[4 * j4], z.x, p0[0]);
-      p0[1] = fmaf(g0[4 * j4 + 1], z.y, p0[1]);
-      p0[2] = fmaf(g0[4 * j4 + 2], z.z, p0[2]);
-      p0[3] = fmaf(g0[4 * j4 + 3], z.w, p0[3]);
-      p1[0] = fmaf(g1[4 * j4], z.x, p1[0]);
-      p1[1] = fmaf(g1[4 * j4 + 1], z.y, p1[1]);
-      p1[2] = fmaf(g1[4 * j4 + 2], z.z, p1[2]);
-      p1[3] = fmaf(g1[4 * j4 + 3], z.w, p1[3]);
+    for (int e = 0; e < NR; e += 4) {               // zeros past n: a test per step would keep
+      const float4 z = v4[e / 4];                   // the loads from overlapping
+      a0 = fmaf(g[e], z.x, a0);
+      a1 = fmaf(g[e + 1], z.y, a1);
+      a0 = fmaf(g[e + 2], z.z, a0);
+      a1 = fmaf(g[e + 3], z.w, a1);
     }
-    __syncwarp();
-    g0o = v0ok ? (p0[0] + p0[1]) + (p0[2] + p0[3]) : 0.f;
-    g1o = v1ok ? (p1[0] + p1[1]) + (p1[2] + p1[3]) : 0.f;
+#pragma unroll
+    for (int e = 0; e < NS; e += 4) {
+      const float4 z = v4[(NR + e) / 4], f = apgdc_sm[e / 4 * threads + slot];
+      a0 = fmaf(f.x, z.x, a0);
+      a1 = fmaf(f.y, z.y, a1);
+      a0 = fmaf(f.z, z.z, a0);
+      a1 = fmaf(f.w, z.w, a1);
+    }
+    float t = a0 + a1;
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    return own ? t : 0.f;
+  };
+  const float bb = own ? a.b[row] : 0.f;
+  float x = own ? a.x[row] : 0.f;
+  int parity = 0;
+  // one sum over the rows of p q, the same in every thread
+  auto block_product_sum = [&](float p, float q) {
+    const float t = pair_product_sum<SMALL>(p, q);
+    if (rows_warp && lane == 0) s_red[parity][0][warp] = t;
+    __syncthreads();
+    const float r = pair_total<GROUPS>(s_red[parity][0]);
+    parity ^= 1;
+    return r;
   };
 
   // ---- Lipschitz constant: Lanczos from the all-ones vector
-  const float vinit = rsqrtf((float)n);
-  float y0 = v0ok ? vinit : 0.f, y1 = v1ok ? vinit : 0.f;   // v_j
-  float z0 = 0.f, z1 = 0.f;                                 // v_{j-1}
-  float theta = 0.f, theta_prev = 0.f, beta_prev = 0.f;
-  int m = 0;
-  for (int j = 0; j < LZ_MAX; ++j) {
-    float g0, g1;
-    gemv(y0, y1, g0, g1);
-    const float alpha = warp_sum(fmaf(y0, g0, y1 * g1));
-    const float w0 = g0 - alpha * y0 - beta_prev * z0;
-    const float w1 = g1 - alpha * y1 - beta_prev * z1;
-    const float beta = sqrtf(fmaxf(warp_sum(fmaf(w0, w0, w1 * w1)), 0.f));
-    if (lane == 0) {
-      s_al[j] = alpha;
-      s_be[j] = beta;
-    }
-    m = j + 1;
-    __syncwarp();
-    const bool last = (m == n) || (m == LZ_MAX) || !(beta > 1e-7f * fabsf(alpha));
-    if (last || (m % 4) == 0) {
-      theta = tridiag_top(s_al, s_be, m, &s_theta);
-      if (last || fabsf(theta - theta_prev) <= LZ_TOL * fabsf(theta)) break;
-      theta_prev = theta;
-    }
-    const float inv = 1.f / beta;
-    z0 = y0;
-    z1 = y1;
-    y0 = w0 * inv;
-    y1 = w1 * inv;
-    beta_prev = beta;
-  }
-  const float L = 1.01f * (theta > 0.f ? theta : 1.f);
-  const float invL = 1.f / L;
-  const float thr = a.lam * invL;
-
-  // ---- monotone FISTA
-  float Gx0, Gx1;
-  gemv(x0, x1, Gx0, Gx1);
-  y0 = x0;
-  y1 = x1;
-  float Gy0 = Gx0, Gy1 = Gx1;
-  float t = 1.f;
-  int it = 0;
-  for (it = 1; it <= a.max_iter; ++it) {
-    const float u0 = y0 - (Gy0 - bb0) * invL, u1 = y1 - (Gy1 - bb1) * invL;
-    float zz0 = a.positive ? fmaxf(u0 - thr, 0.f) : copysignf(fmaxf(fabsf(u0) - thr, 0.f), u0);
-    float zz1 = a.positive ? fmaxf(u1 - thr, 0.f) : copysignf(fmaxf(fabsf(u1) - thr, 0.f), u1);
-    if (!v0ok) zz0 = 0.f;
-    if (!v1ok) zz1 = 0.f;
-    float Gz0, Gz1;
-    gemv(zz0, zz1, Gz0, Gz1);
-    // F(z) - F(x) from the difference itself (see k_apgd_full)
-    const float dF = warp_sum(fmaf(zz0 - x0, 0.5f * (Gz0 + Gx0) - bb0, a.lam * (fabsf(zz0) - fabsf(x0))) +
-                              fmaf(zz1 - x1, 0.5f * (Gz1 + Gx1) - bb1, a.lam * (fabsf(zz1) - fabsf(x1))));
-    const float d0 = zz0 - y0, d1 = zz1 - y1;
-    const float step = sqrtf(warp_sum(fmaf(d0, d0, d1 * d1)));
-    const float nz = sqrtf(warp_sum(fmaf(zz0, zz0, zz1 * zz1)));
-    const float t1 = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
-    const bool accept = dF <= 0.f;
-    const float c1 = t / t1, c2 = (t - 1.f) / t1;
-    const float xn0 = accept ? zz0 : x0, xn1 = accept ? zz1 : x1;
-    const float Gxn0 = accept ? Gz0 : Gx0, Gxn1 = accept ? Gz1 : Gx1;
-    y0 = xn0 + c1 * (zz0 - xn0) + c2 * (xn0 - x0);
-    y1 = xn1 + c1 * (zz1 - xn1) + c2 * (xn1 - x1);
-    Gy0 = Gxn0 + c1 * (Gz0 - Gxn0) + c2 * (Gxn0 - Gx0);
-    Gy1 = Gxn1 + c1 * (Gz1 - Gxn1) + c2 * (Gxn1 - Gx1);
-    x0 = xn0;
-    x1 = xn1;
-    Gx0 = Gxn0;
-    Gx1 = Gxn1;
-    t = t1;
-    if (step <= a.eps * nz) break;
-  }
-  if (it > a.max_iter) it = a.max_iter;
-  // objective of the returned x, in double-float (reported only)
-  const Df xg = warp_df_sum(df_add(df_prod(x0, Gx0), df_prod(x1, Gx1)));
-  const Df bx = warp_df_sum(df_add(df_prod(bb0, x0), df_prod(bb1, x1)));
-  const Df l1 = warp_df_sum(df_add(Df{fabsf(x0), 0.f}, Df{fabsf(x1), 0.f}));
-  const Df Fx = df_add(df_add(df_scale(xg, 0.5f), df_neg(bx)), df_scale(l1, a.lam));
-  if (v0ok) a.x[i0] = x0;
-  if (v1ok) a.x[i1] = x1;
-  if (lane == 0) {
-    if (a.out_iters) *a.out_iters = it;
-    if (a.out_L) *a.out_L = (double)L;
-    if (a.out_F) *a.out_F = (double)Fx.hi + (double)Fx.lo;
-    if (a.out_lanczos) *a.out_lanczos = m;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// One-CTA variant for mid-size supports (WARP_NMAX < n <= CTA_NMAX): the same
-// Lanczos step size, monotone FISTA, stop rule and reported objective, with G
-// cached in shared memory and thread i owning row i of every vector, so the
-// matrix-vector product (thread i: its row of G against the broadcast input)
-// and all elementwise steps need no exchange. A FISTA iteration crosses two
-// block barriers (input vector complete; partial sums complete) instead of a
-// cluster exchange and five barriers.
-constexpr int CTA_NMAX = 224;
-constexpr int CTA_LDG = 228;   // G row stride in floats: 16-byte aligned, 57 x 16 B (odd) so
-                               // eight rows read by a 128-bit phase hit distinct banks
-
-__device__ __forceinline__ float row_dot(const float* __restrict__ Grow, const float* __restrict__ v, int n4) {
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  const float4* g4 = reinterpret_cast<const float4*>(Grow);
-  const float4* v4 = reinterpret_cast<const float4*>(v);
-#pragma unroll 4
-  for (int c = 0; c < n4; ++c) {
-    const float4 g = g4[c], z = v4[c];
-    a0 = fmaf(g.x, z.x, a0);
-    a1 = fmaf(g.y, z.y, a1);
-    a2 = fmaf(g.z, z.z, a2);
-    a3 = fmaf(g.w, z.w, a3);
-  }
-  return (a0 + a1) + (a2 + a3);
-}
-
-// Sum of K per-thread values over the block, the same in every thread (each
-// adds the warps' partials in warp order). buf alternates between two
-// halves, so back-to-back reductions need no extra barrier.
-template <int K>
-__device__ __forceinline__ void cta_sum(float (&v)[K], float* red, int& parity) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int off = 16; off; off >>= 1)
-#pragma unroll
-    for (int q = 0; q < K; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-  float* buf = red + parity * (APGD_THREADS / 32) * 4;
-  parity ^= 1;
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < K; ++q) buf[warp * 4 + q] = v[q];
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < K; ++q) {
-    float t = 0.f;
-    for (int w = 0; w < nw; ++w) t += buf[w * 4 + q];
-    v[q] = t;
-  }
-}
-
-__global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_cta(const __grid_constant__ ApgdBatch batch) {
-  extern __shared__ __align__(16) float apgdc_sm[];
-  __shared__ __align__(16) float vs[CTA_LDG];      // the broadcast input of a product
-  __shared__ float s_red[2 * (APGD_THREADS / 32) * 4];
-  __shared__ Df s_dred[(APGD_THREADS / 32) * 3];
-  __shared__ float s_al[LZ_MAX], s_be[LZ_MAX], s_theta;
-  const ApgdArgs& a = batch.job[blockIdx.x];
-  float* Gc = apgdc_sm;                             // n rows of CTA_LDG floats
-  const int n = a.n, tid = threadIdx.x;
-  const int n4 = (n + 3) >> 2;
-  load_rows_async(Gc, CTA_LDG, a.G, a.ldg, 0, n, n, a.vec_ok != 0);
-  const bool own = tid < n;
-  const float* Grow = Gc + (size_t)(own ? tid : 0) * CTA_LDG;
-  const float bb = own ? a.b[tid] : 0.f;
-  float x = own ? a.x[tid] : 0.f;
-  int parity = 0;
-
-  // ---- Lipschitz constant: Lanczos from the all-ones vector
   float v = own ? rsqrtf((float)n) : 0.f, vprev = 0.f;
-  if (tid < CTA_LDG) vs[tid] = v;
+  for (int i = tid; i < 2 * LDV; i += blockDim.x) vs[i] = 0.f;
+  for (int i = tid; i < 2 * 3 * 16; i += blockDim.x) (&s_red[0][0][0])[i] = 0.f;
+  __syncthreads();
+  if (put) *vrow = v;
   __syncthreads();
   float theta = 0.f, theta_prev = 0.f, beta_prev = 0.f;
   int m = 0;
   for (int j = 0; j < LZ_MAX; ++j) {
-    const float g = own ? row_dot(Grow, vs, n4) : 0.f;
-    float ra[1] = {v * g};
-    cta_sum<1>(ra, s_red, parity);
-    const float alpha = ra[0];
-    const float w = own ? g - alpha * v - beta_prev * vprev : 0.f;
-    float rb[1] = {w * w};
-    cta_sum<1>(rb, s_red, parity);
-    const float beta = sqrtf(fmaxf(rb[0], 0.f));
+    const float gv = product();
+    const float alpha = block_product_sum(v, gv);
+    const float w = own ? gv - alpha * v - beta_prev * vprev : 0.f;
+    const float beta = sqrtf(fmaxf(block_product_sum(w, w), 0.f));
     if (tid == 0) {
       s_al[j] = alpha;
       s_be[j] = beta;
@@ -1070,67 +987,96 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_cta(const __grid_const
       theta_prev = theta;
     }
     vprev = v;
-    v = w / beta;
-    if (own) vs[tid] = v;                           // every read of vs ended before the sums
+    v = SMALL ? w * (1.f / beta) : w / beta;
+    if (put) *vrow = v;                             // every read of vs ended before the sums
     beta_prev = beta;
     __syncthreads();
   }
   const float L = 1.01f * (theta > 0.f ? theta : 1.f);
   const float invL = 1.f / L;
-  const float thr = a.lam * invL;
+  const float thr = __fmul_rn(a.lam, invL);
+  // |u| - lambda / L, in SMALL with one rounding
+  auto shrink = [&](float v) { return fmaxf(SMALL ? fmaf(-a.lam, invL, v) : v - thr, 0.f); };
 
   // ---- initial G x
   __syncthreads();                                  // every read of vs ended
-  if (own) vs[tid] = x;
+  if (put) *vrow = x;
+  if (tid == 0) s_stop = 0;
   __syncthreads();
-  float Gx = own ? row_dot(Grow, vs, n4) : 0.f;
+  float Gx = product();
   float y = x, Gy = Gx;
   __syncthreads();                                  // every read of vs ended
 
   // ---- monotone FISTA
-  float t = 1.f;
+  float t = 1.f;                                    // the last warp's: momentum
   int it = 0;
   for (it = 1; it <= a.max_iter; ++it) {
     const float u = y - (Gy - bb) * invL;
-    float z = a.positive ? fmaxf(u - thr, 0.f) : copysignf(fmaxf(fabsf(u) - thr, 0.f), u);
+    float z = a.positive ? shrink(u) : copysignf(shrink(fabsf(u)), u);
     if (!own) z = 0.f;
-    if (own) vs[tid] = z;                           // the last product's reads ended before its sums
+    if (put) *vrow = z;                             // the last product's reads ended before its sums
     __syncthreads();
-    const float Gz = own ? row_dot(Grow, vs, n4) : 0.f;
-    // F(z) - F(x) from the difference itself (see k_apgd_full)
-    const float d = z - y;
-    float r3[3] = {own ? fmaf(z - x, 0.5f * (Gz + Gx) - bb, a.lam * (fabsf(z) - fabsf(x))) : 0.f, d * d, z * z};
-    cta_sum<3>(r3, s_red, parity);
-    const float step = sqrtf(r3[1]);
-    const float nz = sqrtf(r3[2]);
-    const float t1 = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
-    const bool accept = r3[0] <= 0.f;
-    const float c1 = t / t1, c2 = (t - 1.f) / t1;
-    const float xn = accept ? z : x, Gxn = accept ? Gz : Gx;
-    y = xn + c1 * (z - xn) + c2 * (xn - x);
-    Gy = Gxn + c1 * (Gz - Gxn) + c2 * (Gxn - Gx);
-    x = xn;
-    Gx = Gxn;
-    t = t1;
-    if (step <= a.eps * nz) break;
+    if (s_stop) break;                              // the iteration before was the last one
+    float Gz = 0.f;
+    if (rows_warp) {
+      Gz = product();
+      // F(z) - F(x) from the difference itself (see k_apgd_full); the row's two
+      // threads take a sum each, and share the third
+      const float d = z - y;
+      const float dF = own ? fmaf(z - x, 0.5f * (Gz + Gx) - bb, a.lam * (fabsf(z) - fabsf(x))) : 0.f;
+      const float dd = __fmul_rn(d, d);
+      float r0;
+      if (SMALL) {
+        const float o = __shfl_xor_sync(0xffffffffu, h ? dd : dF, 16);
+        r0 = pair_butterfly(h ? fmaf(d, d, o) : dF + o, false);
+      } else {
+        r0 = pair_butterfly(h ? dd : dF, true);
+      }
+      const float r2 = pair_product_sum<SMALL>(z, z);
+      if (lane < 2) s_red[parity][h][warp] = r0;
+      if (lane == 0) s_red[parity][2][warp] = r2;
+    } else if (lane == 0) {
+      const float t1 = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
+      s_mom = make_float2(t / t1, (t - 1.f) / t1);
+      t = t1;
+    }
+    __syncthreads();
+    if (rows_warp) {
+      const bool accept = pair_total<GROUPS>(s_red[parity][0]) <= 0.f;
+      const float c1 = s_mom.x, c2 = s_mom.y;
+      const float xn = accept ? z : x, Gxn = accept ? Gz : Gx;
+      y = xn + c1 * (z - xn) + c2 * (xn - x);
+      Gy = Gxn + c1 * (Gz - Gxn) + c2 * (Gxn - Gx);
+      x = xn;
+      Gx = Gxn;
+    } else if (lane == 0) {
+      const float step = sqrtf(pair_total<GROUPS>(s_red[parity][1]));
+      const float nz = sqrtf(pair_total<GROUPS>(s_red[parity][2]));
+      s_stop = step <= a.eps * nz;
+    }
+    parity ^= 1;
   }
-  if (it > a.max_iter) it = a.max_iter;
+  it = min(it - 1, a.max_iter);
   // objective of the returned x, in double-float (reported only)
   {
-    const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     Df p[3] = {df_prod(x, Gx), df_prod(bb, x), Df{fabsf(x), 0.f}};
-    for (int off = 16; off; off >>= 1)
+    for (int off = 16; off > 1; off >>= 1)
 #pragma unroll
-      for (int q = 0; q < 3; ++q) p[q] = df_add(p[q], df_shfl_xor(p[q], off));
-    if (lane == 0)
+      for (int i = 0; i < 3; ++i) p[i] = df_add(p[i], df_shfl_xor(p[i], off));
+    if (rows_warp && lane == 0)
 #pragma unroll
-      for (int q = 0; q < 3; ++q) s_dred[warp * 3 + q] = p[q];
+      for (int i = 0; i < 3; ++i) s_dred[warp * 3 + i] = p[i];
     __syncthreads();
     if (tid == 0) {
       Df tot[3] = {};
-      for (int w = 0; w < nw; ++w)
 #pragma unroll
-        for (int q = 0; q < 3; ++q) tot[q] = df_add(tot[q], s_dred[w * 3 + q]);
+      for (int i = 0; i < 3; ++i) {
+        if (SMALL)
+          tot[i] = df_add(df_add(s_dred[i], s_dred[6 + i]), df_add(s_dred[3 + i], s_dred[9 + i]));
+        else
+          for (int w = 0; w < 2 * groups; w += 2)
+            tot[i] = df_add(tot[i], df_add(s_dred[w * 3 + i], s_dred[w * 3 + 3 + i]));
+      }
       const Df Fx = df_add(df_add(df_scale(tot[0], 0.5f), df_neg(tot[1])), df_scale(tot[2], a.lam));
       if (a.out_iters) *a.out_iters = it;
       if (a.out_L) *a.out_L = (double)L;
@@ -1138,8 +1084,13 @@ __global__ void __launch_bounds__(APGD_THREADS, 1) k_apgd_cta(const __grid_const
       if (a.out_lanczos) *a.out_lanczos = m;
     }
   }
-  if (own) a.x[tid] = x;
+  if (put) a.x[row] = x;
 }
+
+// Columns per thread of each instantiation. Registers: 65536 over the block's
+// threads; the largest keeps its last columns in shared memory.
+constexpr int CTA_NC[4] = {32, 64, 96, 112};
+constexpr int CTA_NS = 16;
 
 }  // namespace
 
@@ -1148,35 +1099,38 @@ namespace {
 // Launch shape of one restricted problem: which kernel, cluster size, rows per
 // CTA, whether the CTAs cache their rows of G, dynamic shared memory.
 struct ApgdShape {
-  bool warp = false;   // one-warp kernel (n <= WARP_NMAX)
-  bool cta = false;    // one-CTA kernel (WARP_NMAX < n <= CTA_NMAX)
+  int cta = -1;        // one-CTA kernel (n <= CTA_NMAX): its instantiation (CTA_NC)
   bool full;
   int CS;
   int rows_per;
   int cache;
   int n_pad;
   size_t smem;
+  int threads = APGD_THREADS;
+  bool by_alignment = false;   // k_apgd_full: unaligned rows of G by single columns
 };
 
 // dynamic shared memory ceilings: 227 KB per CTA minus the kernels' static arrays
 constexpr size_t kLimitRows = 200 * 1024;
-constexpr size_t kLimitFull = 226 * 1024;
+constexpr size_t kLimitFull = 231200;
 
 int apgd_setup(int* cs_max_out) {
   static int cs_max = 0;
   static bool attrs_set = false;
   if (cs_max == 0) {
     cudaError_t e1 = cudaFuncSetAttribute(k_apgd, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaError_t e2 = cudaFuncSetAttribute(k_apgd_full, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cs_max = (e1 == cudaSuccess && e2 == cudaSuccess) ? 16 : 8;
+    cudaError_t e2 = cudaFuncSetAttribute(k_apgd_full<APGD_THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e3 =
+        cudaFuncSetAttribute(k_apgd_full<2 * APGD_THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cs_max = (e1 == cudaSuccess && e2 == cudaSuccess && e3 == cudaSuccess) ? 16 : 8;
     cudaGetLastError();
   }
   if (!attrs_set) {
     PC_CUDA(cudaFuncSetAttribute(k_apgd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLimitRows));
-    PC_CUDA(cudaFuncSetAttribute(k_apgd_full, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PC_CUDA(cudaFuncSetAttribute(k_apgd_full<APGD_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kLimitFull));
-    PC_CUDA(cudaFuncSetAttribute(k_apgd_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(float) * CTA_NMAX * CTA_LDG)));
+    PC_CUDA(cudaFuncSetAttribute(k_apgd_full<2 * APGD_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kLimitFull));
     attrs_set = true;
   }
   *cs_max_out = cs_max;
@@ -1185,25 +1139,22 @@ int apgd_setup(int* cs_max_out) {
 
 int apgd_shape(int S, int cs_max, ApgdShape* out) {
   const int n_pad = (S + 3) & ~3;
-  // full-vector kernel: 2 local slices, 2 receive buffers and 6 full vectors
-  // (+ cached rows of G); its slices hold a multiple of 4 rows (bulk copies)
+  // full-vector kernel: 2 receive buffers and 6 full vectors, and as many rows of
+  // G as fit beside them; a CTA's rows are a multiple of 4 (16-byte stores)
   auto rows_full = [&](int cs) { return (ceil_div(S, cs) + 3) & ~3; };
-  auto bytes_full = [&](int cs, bool cached) {
-    const size_t rp = (size_t)rows_full(cs);
-    return sizeof(float) * (2 * rp + 8 * (size_t)n_pad) + (cached ? sizeof(float) * rp * n_pad : 0);
-  };
+  const size_t vec_full = sizeof(float) * 8 * (size_t)n_pad, row_full = sizeof(float) * (size_t)n_pad;
   // row-slice kernel (larger supports): one full vector + 8 row slices
   auto bytes_rows = [&](int cs, bool cached) {
     const size_t rp = (size_t)ceil_div(S, cs);
     return sizeof(float) * ((size_t)n_pad + 8 * rp) + 16 + 16 * sizeof(Df) +
            (cached ? sizeof(float) * rp * n_pad : 0);
   };
-  // cluster size: the smallest power of two whose CTAs each cache at most
-  // ~64 KB of G in shared memory (a matrix-vector product then streams it in
-  // ~500 cycles), else the smallest that caches G at all, else cs_max
+  // cluster size: the smallest power of two whose CTAs each hold at most 32 KB of
+  // G (a matrix-vector product then streams it in ~250 cycles), else cs_max
   ApgdShape sh;
-  if (S <= WARP_NMAX) {
-    sh.warp = true;
+  if (S <= CTA_NMAX) {
+    sh.cta = 0;
+    while (S > 2 * CTA_NC[sh.cta]) ++sh.cta;
     sh.full = true;
     sh.CS = 1;
     sh.cache = 1;
@@ -1213,27 +1164,29 @@ int apgd_shape(int S, int cs_max, ApgdShape* out) {
     *out = sh;
     return PC_OK;
   }
-  if (S <= CTA_NMAX) {
-    sh.cta = true;
-    sh.full = true;
-    sh.CS = 1;
-    sh.cache = 1;
-    sh.smem = sizeof(float) * (size_t)S * CTA_LDG;
-    sh.rows_per = S;
-    sh.n_pad = n_pad;
-    *out = sh;
-    return PC_OK;
-  }
   sh.full = true;
   sh.CS = 1;
-  const size_t share_target = 64 * 1024;
-  while (sh.CS < cs_max && (bytes_full(sh.CS, true) > kLimitFull ||
-                            sizeof(float) * (size_t)rows_full(sh.CS) * n_pad > share_target))
-    sh.CS *= 2;
-  sh.cache = bytes_full(sh.CS, true) <= kLimitFull ? 1 : 0;
-  sh.smem = bytes_full(sh.CS, sh.cache != 0);
-  if (sh.smem > kLimitFull) {
+  const size_t share_target = 32 * 1024;
+  while (sh.CS < cs_max && rows_full(sh.CS) * row_full > share_target) sh.CS *= 2;
+  // rows of G in shared memory: all, else as many as fit if that is half of them,
+  // else 170 KB, which leaves the rows read from L2 a first-level cache to arrive in
+  // (2500 atoms, 225 KB: 19.6 us an iteration, 170 KB 16.0; 900 atoms 3.76 and 4.09).
+  // With rows to read 16 warps multiply, not 8 (1300 atoms 6.6 and 5.7 us).
+  auto fit = [&](size_t lim) { return lim > vec_full ? (int)((lim - vec_full) / row_full) & ~3 : 0; };
+  const int rp = rows_full(sh.CS);
+  sh.cache = std::min(rp, fit(kLimitFull));
+  if (sh.cache < rp) {
+    sh.threads = 2 * APGD_THREADS;
+    if (2 * sh.cache < rp) sh.cache = fit(170 * 1024);
+    // a lane's columns, hence the order of its sum, go by the alignment of the rows
+    // unless 226 KB hold all of them beside the vectors and two slices
+    sh.by_alignment = 2 * sizeof(float) * rp + vec_full + rp * row_full > 226 * 1024;
+  }
+  sh.smem = vec_full + sh.cache * row_full;
+  if (2 * sizeof(float) * rp + vec_full > 226 * 1024) {
     sh.full = false;
+    sh.threads = APGD_THREADS;
+    sh.by_alignment = false;
     sh.CS = 1;
     while (sh.CS < cs_max && bytes_rows(sh.CS, true) > kLimitRows) sh.CS *= 2;
     if (bytes_rows(sh.CS, false) > kLimitRows)
@@ -1267,6 +1220,7 @@ ApgdArgs make_args(const ApgdJob& j, const ApgdShape& sh) {
   a.n_pad = sh.n_pad;
   a.cache = sh.cache;
   a.vec_ok = ((j.ldg & 3) == 0 && (reinterpret_cast<uintptr_t>(j.G) & 15) == 0) ? 1 : 0;
+  a.scalar = sh.by_alignment && !a.vec_ok;
   return a;
 }
 
@@ -1287,33 +1241,37 @@ int run_apgd_jobs(const ApgdJob* jobs, int n_jobs, cudaStream_t st) {
     ApgdBatch batch{};
     size_t smem = 0;
     const bool full = shapes[i].full;
-    const bool warp = shapes[i].warp, cta = shapes[i].cta;
+    const int cta = shapes[i].cta;
+    int rows = 0;
     const int CS = shapes[i].CS;
     for (int j = i; j < n_jobs && batch.n_jobs < APGD_BATCH_MAX; ++j) {
-      if (done[j] || shapes[j].full != full || shapes[j].CS != CS || shapes[j].warp != warp ||
-          shapes[j].cta != cta)
+      if (done[j] || shapes[j].full != full || shapes[j].CS != CS || shapes[j].cta != cta ||
+          shapes[j].threads != shapes[i].threads)
         continue;
       batch.job[batch.n_jobs++] = make_args(jobs[j], shapes[j]);
       smem = std::max(smem, shapes[j].smem);
+      rows = std::max(rows, jobs[j].n);
       done[j] = 1;
     }
-    if (warp) {
+    if (cta >= 0) {
       ProfScope prof_scope_(PROF_APGD, st);
       prof_scope_.kernels = 1;
-      k_apgd_warp<<<batch.n_jobs, 32, 0, st>>>(batch);
-      PC_LAUNCH_CHECK();
-      continue;
-    }
-    if (cta) {
-      ProfScope prof_scope_(PROF_APGD, st);
-      prof_scope_.kernels = 1;
-      k_apgd_cta<<<batch.n_jobs, APGD_THREADS, smem, st>>>(batch);
+      // two threads a row, whole groups of 32 rows (64 of the smallest), and the last warp
+      const int rt = cta == 0 ? 2 * WARP_NMAX : 64 * ceil_div(rows, 32), threads = rt + 32;
+      if (cta == 0)
+        k_apgd_cta<CTA_NC[0], 0><<<batch.n_jobs, threads, 0, st>>>(batch);
+      else if (cta == 1)
+        k_apgd_cta<CTA_NC[1], 0><<<batch.n_jobs, threads, 0, st>>>(batch);
+      else if (cta == 2)
+        k_apgd_cta<CTA_NC[2], 0><<<batch.n_jobs, threads, 0, st>>>(batch);
+      else
+        k_apgd_cta<CTA_NC[3], CTA_NS><<<batch.n_jobs, threads, sizeof(float) * CTA_NS * rt, st>>>(batch);
       PC_LAUNCH_CHECK();
       continue;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CS * batch.n_jobs, 1, 1);
-    cfg.blockDim = dim3(APGD_THREADS, 1, 1);
+    cfg.blockDim = dim3(shapes[i].threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -1327,7 +1285,9 @@ int run_apgd_jobs(const ApgdJob* jobs, int n_jobs, cudaStream_t st) {
     {
       ProfScope prof_scope_(PROF_APGD, st);
       prof_scope_.kernels = 1;
-      e = full ? cudaLaunchKernelEx(&cfg, k_apgd_full, batch) : cudaLaunchKernelEx(&cfg, k_apgd, batch);
+      e = !full                                ? cudaLaunchKernelEx(&cfg, k_apgd, batch)
+          : shapes[i].threads == APGD_THREADS ? cudaLaunchKernelEx(&cfg, k_apgd_full<APGD_THREADS>, batch)
+                                              : cudaLaunchKernelEx(&cfg, k_apgd_full<2 * APGD_THREADS>, batch);
     }
     PC_CUDA(e);
   }
