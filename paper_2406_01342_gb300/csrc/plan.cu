@@ -86,9 +86,9 @@ static void psi_hat_grid(int n, int G, int W, const std::vector<double>& wz, con
   for (double& v : out) v *= W;
 }
 
-// Chebyshev coefficients in y = 2 (t / T)^2 - 1 of 1 / psi(t), |t| <= T = 1/4: the
-// w-kernel's correction as a polynomial (psi is entire and even: 16 terms leave
-// 1e-12).
+// Chebyshev coefficients in y = 2 (t / T)^2 - 1 of 1 / psi(t), |t| <= T: the
+// w-kernel's correction as a polynomial (psi is entire and even, its first zero
+// past 0.7: 16 terms leave 1e-12 at T = 1/4 and 1e-10 at T = 0.4).
 constexpr int kPsiTerms = 16;
 static void psi_poly(double T, int W, const std::vector<double>& wz, const std::vector<double>& wphi, double* c) {
   double f[kPsiTerms];
@@ -359,7 +359,7 @@ __global__ void k_slot_gather(const double* __restrict__ uvw, const unsigned* __
 }
 
 struct PixGeom {
-  double dl, w0, dw, s_c, beta;
+  double dl, w0, dw, s_c, inv_t;   // inv_t: 1 / T of psi_poly
   int N, W;
   bool wstack;
 };
@@ -391,7 +391,7 @@ __global__ void k_pix_tab(PixGeom g, const double* __restrict__ rpsi, const doub
   double t = 0.0, rw = 1.0;
   if (g.wstack) {
     t = g.dw * (s - g.s_c);
-    const double y = 32.0 * t * t - 1.0;            // 2 (t / T)^2 - 1, T = 1/4
+    const double z = t * g.inv_t, y = 2.0 * z * z - 1.0;
     double b1 = 0.0, b2 = 0.0;
 #pragma unroll
     for (int k = kPsiTerms - 1; k >= 1; --k) {
@@ -764,11 +764,22 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   p->logG = 0;
   while ((1 << p->logG) < p->G) ++p->logG;
   p->nT = p->G / p->T;
+  // the kernel's shape: 2.30 W suits an oversampling of 2; a smaller image's is a
+  // little more (pi (1 - 1 / 2 sigma) W, as for that 2.30)
   p->beta = 2.30 * p->W;
+  if (p->resample.K > 0)
+    p->beta = 0.976 * M_PI * (1.0 - 0.5 / std::min(2.3, p->resample.G * p->resample.d / N)) * p->W;
   const double half = 0.5 * Nt * dlt;
   const double r2c = 2.0 * half * half;
   const double s_min = -r2c / (1.0 + std::sqrt(1.0 - r2c));
   const double s_max = 0.0;
+  // The planes are spaced for the corner of the transforms' image but centred on the
+  // N x N pixels' own range, which then is sampled more finely than at 2; only the
+  // rim that the interpolation's outer taps touch lies beyond 1/4 (figures at
+  // choose_resample).
+  const double half_n = 0.5 * N * p->dl, r2n = 2.0 * half_n * half_n;
+  const double s_min_n = -r2n / (1.0 + std::sqrt(1.0 - r2n));
+  double t_max = 0.25;
   p->phase = phase_scale(std::max(std::fabs(p->w_min), std::fabs(p->w_max)), -s_min);
   if (M > 0 && p->w_max > p->w_min) {
     p->wstack = true;
@@ -779,7 +790,8 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
                   max_planes);
     p->P = (int)planes;
     p->w0 = p->w_min - 0.5 * p->W * p->dw;
-    p->s_c = 0.5 * (s_min + s_max);
+    p->s_c = 0.5 * (s_min_n + s_max);
+    t_max = std::max(p->dw * std::max(p->s_c - s_min, s_max - p->s_c), 0.25);
   } else {
     p->wstack = false;
     p->P = 1;
@@ -806,14 +818,14 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   for (double& v : rpsi) v = 1.0 / v;
   rpsi.resize(rpsi.size() + kPsiTerms);
   double* poly = rpsi.data() + Nt / 2 + 1;
-  psi_poly(0.25, p->W, wz, wphi, poly);
+  psi_poly(t_max, p->W, wz, wphi, poly);
   double* d_psi;
   PC_TRY(tmp.alloc((void**)&d_psi, sizeof(double) * rpsi.size()));
   PC_TRY(up.upload(d_psi, rpsi.data(), sizeof(double) * rpsi.size()));
   const int64_t NN = (int64_t)N * N, NNt = (int64_t)Nt * Nt;
   PC_TRY(dev_alloc_t(p, &p->pix_tab, NNt));
   {
-    PixGeom pg{dlt, p->w0, p->dw, p->s_c, p->beta, Nt, p->W, p->wstack};
+    PixGeom pg{dlt, p->w0, p->dw, p->s_c, 1.0 / t_max, Nt, p->W, p->wstack};
     k_pix_tab<<<dim3(ceil_div(Nt / 2 + 1, 128), Nt / 2 + 1), 128, 0, st>>>(pg, d_psi, d_psi + Nt / 2 + 1, p->pix_tab);
     PC_LAUNCH_CHECK();
   }

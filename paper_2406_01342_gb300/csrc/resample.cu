@@ -173,18 +173,23 @@ int apply(const float* in, int n_in, int n_cols, const BandTable& t, float* out,
 
 // The smallest grid of side 512 or more whose image of side G / 2 still samples
 // the visibilities: with K taps (16 .. 40) past the field's edge the pixels are d
-// = N / (G / 2 - K) wide, and K must reach beta = 14.9. turns: the most that a
-// visibility turns per image pixel, w-term included. Only grids of side 2048 and
-// more are replaced: at 1024 the passes take 28 us of a 512 x 512 certificate's
+// = N / (G / 2 - K) wide, and K must reach beta = 14.9. The small grid oversamples
+// the pixels' field as much as the image's own grid does, up to 2.12: past that
+// the planes cost more than the accuracy gives (1100 x 1100 at 2.05 / 2.12 / 2.3:
+// errors 9.5e-7 / 6.7e-7 / 5.0e-7, against 7.2e-7 on the image's own grid; at 2.3 a
+// quarter more planes). turns: the most that a visibility turns per image pixel,
+// w-term included. Only grids of side 2048 and more are replaced: at 1024 the passes take 28 us of a 512 x 512 certificate's
 // 220, which the interpolation and a wider field's further w-planes would eat.
 Resample choose_resample(int N, int G, double turns) {
   Resample r;
   r.Nt = N;
   r.G = G;
   if (G < 2048) return r;
+  const double sigma = std::min(2.12, (double)G / N);
   for (int g = 512; g < G; g *= 2)
     for (int K = 16; K <= 40; K += 8) {
-      const double d = (double)N / (g / 2 - K), nu = turns * d, beta = M_PI * K * (0.5 - nu);
+      const double d = std::max((double)N / (g / 2 - K), sigma * N / g);
+      const double nu = turns * d, beta = M_PI * K * (0.5 - nu);
       if (d < 1.0 || beta < 14.9) continue;
       r.K = K;
       r.Nt = g / 2;
