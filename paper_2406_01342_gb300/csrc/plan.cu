@@ -86,20 +86,29 @@ static void psi_hat_grid(int n, int G, int W, const std::vector<double>& wz, con
   for (double& v : out) v *= W;
 }
 
-// Chebyshev coefficients in y = 2 (t / T)^2 - 1 of 1 / psi(t), |t| <= T: the
-// w-kernel's correction as a polynomial (psi is entire and even, its first zero
-// past 0.7: 16 terms leave 1e-12 at T = 1/4 and 1e-10 at T = 0.4).
+// 1 / psi(t), |t| <= T, as a polynomial in y = 2 (t / T)^2 - 1: the w-kernel's
+// correction, interpolated at Chebyshev nodes (psi is entire and even, its first
+// zero past 0.7: 16 terms leave 1e-12 at T = 1/4 and 1e-10 at T = 0.4) and
+// turned into powers of y for a Horner sum.
 constexpr int kPsiTerms = 16;
 static void psi_poly(double T, int W, const std::vector<double>& wz, const std::vector<double>& wphi, double* c) {
   double f[kPsiTerms];
   for (int i = 0; i < kPsiTerms; ++i) {
     const double y = std::cos(M_PI * (i + 0.5) / kPsiTerms);
     f[i] = 1.0 / psi_hat_host(T * std::sqrt(0.5 * (y + 1.0)), W, wz, wphi);
+    c[i] = 0.0;
   }
+  double prev[kPsiTerms] = {}, cur[kPsiTerms] = {1.0};   // powers of T_{k-1} and T_k
   for (int k = 0; k < kPsiTerms; ++k) {
     double v = 0.0;
     for (int i = 0; i < kPsiTerms; ++i) v += f[i] * std::cos(M_PI * k * (i + 0.5) / kPsiTerms);
-    c[k] = v * (k ? 2.0 : 1.0) / kPsiTerms;
+    v *= (k ? 2.0 : 1.0) / kPsiTerms;
+    for (int i = 0; i <= k; ++i) c[i] += v * cur[i];
+    for (int i = std::min(k + 1, kPsiTerms - 1); i >= 0; --i) {   // T_{k+1} = 2 y T_k - T_{k-1} (T_1 = y)
+      const double next = (k ? 2.0 : 1.0) * (i ? cur[i - 1] : 0.0) - prev[i];
+      prev[i] = cur[i];
+      cur[i] = next;
+    }
   }
 }
 
@@ -384,28 +393,25 @@ __global__ void k_pix_tab(PixGeom g, const double* __restrict__ rpsi, const doub
                           float4* __restrict__ out) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
   if (b > g.N / 2) return;
-  double l = a * g.dl, m = b * g.dl;
-  double r2 = l * l + m * m;
-  double n = sqrt(1.0 - r2);
-  double s = -r2 / (1.0 + n);        // n - 1 without cancellation
+  const double l = a * g.dl, m = b * g.dl;
+  const double q = 1.0 - (l * l + m * m);
+  // 1 / n = q^(-1/2): an FP32 value and one Newton step (1e-13 relative)
+  double rn = (double)rsqrtf((float)q);
+  rn *= fma(-0.5 * q * rn, rn, 1.5);
+  const double s = q * rn - 1.0;     // n - 1
   double t = 0.0, rw = 1.0;
   if (g.wstack) {
     t = g.dw * (s - g.s_c);
     const double z = t * g.inv_t, y = 2.0 * z * z - 1.0;
-    double b1 = 0.0, b2 = 0.0;
+    rw = poly[kPsiTerms - 1];
 #pragma unroll
-    for (int k = kPsiTerms - 1; k >= 1; --k) {
-      const double v = 2.0 * y * b1 - b2 + poly[k];
-      b2 = b1;
-      b1 = v;
-    }
-    rw = y * b1 - b2 + poly[0];
+    for (int k = kPsiTerms - 2; k >= 0; --k) rw = fma(rw, y, poly[k]);
   }
   double ct = g.w0 * s;
   ct -= rint(ct);                    // exact reduction to [-1/2, 1/2] turns in FP64
   float snf, csf;                    // then an FP32 sine / cosine (~1e-7): FP64 ones are slow here
   sincospif(2.0f * (float)ct, &snf, &csf);
-  const double d = rpsi[a] * rpsi[b] * rw / n;
+  const double d = rpsi[a] * rpsi[b] * rw * rn;
   const float t_hi = (float)t;
   const float4 v = make_float4((float)((double)csf * d), (float)((double)snf * d), t_hi, (float)(t - (double)t_hi));
   write_quadrant(out, g.N, a, b, [&](int, int) { return v; });
