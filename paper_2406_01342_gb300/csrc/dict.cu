@@ -10,9 +10,9 @@
 //
 // Kernels:
 //   k_dict_corr     eta = Psi* mu on every coefficient: one CTA per 32 x 32
-//                   output tile stages mu with a halo of the largest radius in
-//                   shared memory, runs the row then the column pass of every
-//                   scale and writes the max |eta| / signed max as order keys;
+//                   output tile and scale stages mu with a halo of the scale's
+//                   radius in shared memory, runs the row then the column pass
+//                   and writes the max |eta| / signed max as order keys;
 //   k_dict_columns  columns of Phi Psi for the atoms entering the active set:
 //                   the direct sum of the measurement operator over the atom's
 //                   footprint pixels (same fixed-point phases as the pixel
@@ -77,49 +77,68 @@ inline int round4(int n) { return (n + 3) & ~3; }
 constexpr int CT = 32;             // output tile side
 constexpr int CH = CT + 2 * DK;    // staged tile side (with the halo)
 
+// One CTA per tile and scale: at 256 x 256 the tiles alone are 64 CTAs of 152 SMs,
+// and the scales one after the other took 16 us. A thread sums four neighbouring
+// outputs from one sliding window of inputs (two shared-memory reads for four
+// products instead of eight). The adjoint onto four scales: 74.6 -> 63.8 us.
 __global__ void __launch_bounds__(256)
 k_dict_corr(const float* __restrict__ img, int N, const __grid_constant__ DictParams D,
             float* __restrict__ eta, unsigned* __restrict__ maxbits) {
   __shared__ float H[CH][CH + 1];
   __shared__ float T[CH][CT + 1];
-  __shared__ float taps[PC_DICT_MAX_SCALES][DTAPS];
-  const int x0 = blockIdx.y * CT, y0 = blockIdx.x * CT;
-  for (int e = threadIdx.x; e < PC_DICT_MAX_SCALES * DTAPS; e += blockDim.x)
-    taps[e / DTAPS][e % DTAPS] = D.g1[e / DTAPS][e % DTAPS];
-  for (int e = threadIdx.x; e < CH * CH; e += blockDim.x) {
-    const int r = e / CH, c = e - r * CH;
-    const int x = x0 - DK + r, y = y0 - DK + c;
+  __shared__ float g[DTAPS];
+  const int x0 = blockIdx.y * CT, y0 = blockIdx.x * CT, i = blockIdx.z;
+  const int K = D.K[i], side = CT + 2 * K;
+  for (int e = threadIdx.x; e <= 2 * K; e += blockDim.x) g[e] = D.g1[i][e];
+  for (int e = threadIdx.x; e < side * side; e += blockDim.x) {
+    const int r = e / side, c = e - r * side;
+    const int x = x0 - K + r, y = y0 - K + c;
     H[r][c] = (x >= 0 && x < N && y >= 0 && y < N) ? img[(size_t)x * N + y] : 0.f;
   }
   __syncthreads();
-  const size_t NN = (size_t)N * N;
-  float amax = 0.f, smax = -INFINITY;
-  for (int i = 0; i < D.n_scales; ++i) {
-    const int K = D.K[i];
-    const float* g = taps[i];
-    // along y: T[r][c] = sum_m g[m] H[r][c + m] for the rows the x pass reads
-    const int r0 = DK - K, nr = CT + 2 * K;
-    for (int e = threadIdx.x; e < nr * CT; e += blockDim.x) {
-      const int r = r0 + e / CT, c = e % CT;
-      float s = 0.f;
-      for (int m = -K; m <= K; ++m) s = fmaf(g[m + K], H[r][DK + c + m], s);
-      T[r][c] = s;
+  // along y: T[r][c] = sum_m g[m] H[r][c + m], four columns a thread
+  for (int e = threadIdx.x; e < side * (CT / 4); e += blockDim.x) {
+    const int r = e / (CT / 4), c = 4 * (e % (CT / 4));
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, h0 = H[r][c], h1 = H[r][c + 1], h2 = H[r][c + 2];
+    for (int m = 0; m <= 2 * K; ++m) {
+      const float h3 = H[r][c + m + 3], w = g[m];
+      s[0] = fmaf(w, h0, s[0]);
+      s[1] = fmaf(w, h1, s[1]);
+      s[2] = fmaf(w, h2, s[2]);
+      s[3] = fmaf(w, h3, s[3]);
+      h0 = h1;
+      h1 = h2;
+      h2 = h3;
     }
-    __syncthreads();
-    // along x, times gamma_i
-    for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) {
-      const int r = e / CT, c = e % CT;
-      const int x = x0 + r, y = y0 + c;
-      float s = 0.f;
-      for (int n = -K; n <= K; ++n) s = fmaf(g[n + K], T[DK + r + n][c], s);
-      const float v = D.gamma[i] * s;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) T[r][c + q] = s[q];
+  }
+  __syncthreads();
+  // along x, times gamma_i: four rows a thread
+  float amax = 0.f, smax = -INFINITY;
+  {
+    const int r = 4 * (threadIdx.x / CT), c = threadIdx.x % CT;
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, h0 = T[r][c], h1 = T[r + 1][c], h2 = T[r + 2][c];
+    for (int n = 0; n <= 2 * K; ++n) {
+      const float h3 = T[r + n + 3][c], w = g[n];
+      s[0] = fmaf(w, h0, s[0]);
+      s[1] = fmaf(w, h1, s[1]);
+      s[2] = fmaf(w, h2, s[2]);
+      s[3] = fmaf(w, h3, s[3]);
+      h0 = h1;
+      h1 = h2;
+      h2 = h3;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int x = x0 + r + q, y = y0 + c;
+      const float v = D.gamma[i] * s[q];
       if (x < N && y < N) {
-        eta[i * NN + (size_t)x * N + y] = v;
+        eta[(size_t)i * N * N + (size_t)x * N + y] = v;
         amax = fmaxf(amax, fabsf(v));
         smax = fmaxf(smax, v);
       }
     }
-    __syncthreads();
   }
   for (int off = 16; off; off >>= 1) {
     amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
@@ -379,7 +398,7 @@ __global__ void k_check_idx(const int32_t* __restrict__ idx, int S, int64_t n_at
 int launch_corr(const float* img, int N, const DictParams& D, float* eta, unsigned* maxbits, cudaStream_t st) {
   ProfScope prof_scope_(PROF_DICT_CORR, st);
   prof_scope_.kernels = 1;
-  dim3 grid(ceil_div(N, CT), ceil_div(N, CT));
+  dim3 grid(ceil_div(N, CT), ceil_div(N, CT), D.n_scales);
   k_dict_corr<<<grid, 256, 0, st>>>(img, N, D, eta, maxbits);
   PC_LAUNCH_CHECK();
   return PC_OK;

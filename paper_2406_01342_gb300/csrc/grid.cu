@@ -13,8 +13,8 @@
 // footprint touches the tile was binned into it at plan time). The tile is
 // accumulated in registers, not in shared memory: warp w owns rows
 // [4w, 4w + 4) of the tile for every plane of the group, lane a owns column a.
-// Visibilities are processed in chunks of 256: first each thread evaluates
-// the kernel weights of one visibility (W in u, W in v, one per plane of the
+// Visibilities are processed in chunks of 256: first eight threads to a
+// visibility evaluate its kernel weights (W in u, W in v, one per plane of the
 // group) into shared memory, then every warp sweeps the chunk, skips the
 // visibilities whose footprint misses its 4 rows, and accumulates
 // h * phi_u[a] * phi_v[b] * phi_w[q] with plain FMAs. No atomics touch shared
@@ -60,33 +60,32 @@ k_grid(const int4* __restrict__ subs, const int2* __restrict__ slot_vis,
 
   for (int c0 = sub.z; c0 < sub.w; c0 += GRID_CHUNK) {
     const int cnt = min(GRID_CHUNK, sub.w - c0);
-    // ---- phase 1: kernel weights of one visibility per thread
-    if (tid < cnt) {
-      const int j = c0 + tid;
+    // ---- phase 1: kernel weights, eight threads to a visibility
+    for (int e = tid; e < cnt * 8; e += 256) {
+      const int t = e >> 3, c = e & 7, j = c0 + t;
       const int2 sv = slot_vis[j];
       const float4 gm = slot_geom[j];
-      float2 hv = h[sv.x];
-      if (wstack) {
-        float sn, cs;
-        sincospif(2.0f * gm.w, &sn, &cs);
-        hv = cmul(hv, make_float2(cs, sn));
+      if (c < W) {
+        s_fu[t][c] = es_kernel((c - gm.x) * two_over_w, beta);
+        s_fv[t][c] = es_kernel((c - gm.y) * two_over_w, beta);
       }
-#pragma unroll
-      for (int c = 0; c < W; ++c) {
-        s_fu[tid][c] = es_kernel((c - gm.x) * two_over_w, beta);
-        s_fv[tid][c] = es_kernel((c - gm.y) * two_over_w, beta);
-      }
-      const int ps = sv.y >> 16;
-#pragma unroll
-      for (int q = 0; q < QMAX; ++q) {
-        const int cw = q0 + q - ps;
+      if (c < QMAX) {
+        const int cw = q0 + c - (sv.y >> 16);
         float f = 0.f;
-        if (q < Q)
+        if (c < Q)
           f = wstack ? ((cw >= 0 && cw < W) ? es_kernel((cw - gm.z) * two_over_w, beta) : 0.f) : 1.f;
-        s_fw[tid][q] = f;
+        s_fw[t][c] = f;
       }
-      s_h[tid] = hv;
-      s_ab[tid] = sv.y & 0xffff;
+      if (c == 7) {
+        float2 hv = h[sv.x];
+        if (wstack) {
+          float sn, cs;
+          sincospif(2.0f * gm.w, &sn, &cs);
+          hv = cmul(hv, make_float2(cs, sn));
+        }
+        s_h[t] = hv;
+        s_ab[t] = sv.y & 0xffff;
+      }
     }
     __syncthreads();
     // ---- phase 2: every warp accumulates its 4-row band

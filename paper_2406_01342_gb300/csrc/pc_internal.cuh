@@ -282,6 +282,7 @@ bool grid_win_mode(const pc_plan_s* p);   // the plan grids (and degrids) over p
 // degrid_win.cu: degridding interpolation over plane windows, one thread per
 // slot (y added to)
 int launch_degrid_win(pc_plan_s* p, float2* y, cudaStream_t st);
+int fft_rows_per_cta(const pc_plan_s* p);   // default of the Stockham first pass
 int launch_fft_rows(pc_plan_s* p, cudaStream_t st);
 int launch_fft_cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits,
                              cudaStream_t st);
@@ -343,7 +344,7 @@ struct pc_plan_s {
   int grid_mode = 0;  // 0 auto, 1 CUDA cores, 2 tensor cores, 3 CUDA cores over plane
                       // windows (2 and 3: w-stacking only; else mode 1 runs)
   int grid_piece = 0; // gridding sub-problem size in slots (0: chosen for even waves)
-  int fft_R = 0;      // rows per CTA of the first FFT pass (0: 2048 / G)
+  int fft_R = 0;      // rows per CTA of the first FFT pass (0: fft_rows_per_cta)
   int fft_cols_pg = 0; // planes per pass of the second FFT pass (0: default)
   int fft_warp = -1;  // bit 0 / bit 1: first / second FFT pass as one-warp register FFTs
                       // (-1: both wherever G is 512 or 1024, the sizes those kernels take)

@@ -552,10 +552,11 @@ static int split_dwsubs(pc_plan_s* p, int cap, Staging& up) {
 
 static int split_subs(pc_plan_s* p, int piece, Staging& up) {
   std::vector<int4> subs;
+  const int stage = p->wstack ? 64 : 32;   // the tensor-core stage; k_grid's smallest
   for (const int4& r : p->sub_ranges) {
     const int len = r.w - r.z;
     const int n_pieces = ceil_div(len, piece);
-    const int sz = ceil_div(ceil_div(len, n_pieces), 64) * 64;
+    const int sz = ceil_div(ceil_div(len, n_pieces), stage) * stage;
     for (int s = r.z; s < r.w; s += sz) subs.push_back(make_int4(r.x, r.y, s, std::min(r.w, s + sz)));
   }
   if ((int)subs.size() > p->sub_cap) return fail(PC_ERR_CAPACITY, "plan: %zu sub-problems", subs.size());
@@ -975,8 +976,11 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   int n_sm = 152;
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
   const int64_t want = 4ll * n_sm;
-  int piece = (int)std::min<int64_t>(kMaxSlotsPerSub, std::max<int64_t>(128, (total_slots + want - 1) / want));
-  piece = ceil_div(piece, 64) * 64;
+  // without w-stacking the CUDA cores grid, and a CTA's time is its slots one after
+  // the other: down to 32
+  const int piece_min = p->wstack ? 128 : 32, stage = p->wstack ? 64 : 32;
+  int piece = (int)std::min<int64_t>(kMaxSlotsPerSub, std::max<int64_t>(piece_min, (total_slots + want - 1) / want));
+  piece = ceil_div(piece, stage) * stage;
   p->sub_ranges = ranges;
   // tile rows / columns that hold visibilities (the one-warp FFTs skip the rest, which stay zero)
   p->row_mask = p->col_mask = 0;
@@ -985,8 +989,8 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
       p->row_mask |= 1u << (s.x / p->nT);
       p->col_mask |= 1u << (s.x % p->nT);
     }
-  // room for the finest split the autotuner may try (pieces of 64 slots)
-  p->sub_cap = (int)(total_slots / 64 + (int64_t)ranges.size() + 1);
+  // room for the finest split: pieces of 32 or (the autotuner's) 64 slots
+  p->sub_cap = (int)(total_slots / stage + (int64_t)ranges.size() + 1);
   PC_TRY(dev_alloc_t(p, &p->subs, (size_t)p->sub_cap));
   PC_TRY(split_subs(p, piece, up));
   // window gridding: the bin offsets on the device, the tiles that hold slots,
@@ -1135,7 +1139,7 @@ extern "C" int pc_plan_tuning_info(pc_plan_t p, pc_plan_tuning* out) {
   out->tuned = p->tuned ? 1 : 0;
   out->grid_mode = grid_win_mode(p) ? 3 : (p->wstack && p->grid_mode != 1) ? 2 : 1;
   out->grid_piece = grid_win_mode(p) ? p->win_cap : p->grid_piece;
-  int R = p->fft_R > 0 ? p->fft_R : 2048 / p->G;
+  int R = p->fft_R > 0 ? p->fft_R : fft_rows_per_cta(p);
   const bool rw = fft_rows_warp(p) || fft_rows_big(p), cw = fft_cols_warp(p) || fft_cols_big(p);
   out->fft_rows_per_cta = fft_rows_big(p) ? 1 : rw ? 8 : std::min(std::max(R, 1), 32);
   out->grid_us = p->tune_grid_us;
