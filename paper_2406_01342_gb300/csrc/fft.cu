@@ -22,6 +22,8 @@
 // Otherwise, and where the autotuner measured it faster, they run radix-4
 // (plus one radix-2) Stockham stages in shared memory with a twiddle table
 // e^{+2 pi i k / G}.
+#include <climits>
+
 #include "pc_internal.cuh"
 #include "fft.cuh"
 #include "fft_warp.cuh"
@@ -395,8 +397,17 @@ static int cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits
     return launch_fft_cols_big(p, mu, scale, maxbits, st);
   }
   if (fft_cols_warp(p)) {
-    int wpr = 8;                                   // warps per image row: a power of 2 <= P
-    while (wpr > p->P) wpr >>= 1;
+    // warps per image row, a power of 2 <= P: the least planes one after the other in
+    // whole waves of two CTAs on each of 152 SMs (nine planes on eight warps take two
+    // rounds, the second with one warp at work)
+    int wpr = 1, best = INT_MAX;
+    for (int w = 8; w >= 1; w >>= 1) {
+      const int t = ceil_div(ceil_div(p->Nt, 8 / w), 2 * 152) * ceil_div(p->P, w);
+      if (w <= p->P && t < best) {
+        best = t;
+        wpr = w;
+      }
+    }
     const int rpc = 8 / wpr;
     const int ws = p->wstack ? 1 : 0;
     const bool one = wpr == p->P;                  // every warp exactly one plane
