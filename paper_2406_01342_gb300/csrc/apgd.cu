@@ -14,9 +14,10 @@
 // linearly, so the 1 % margin of L covers the remaining error many times.
 //
 // GB300 mapping: one CTA up to 224 atoms (k_apgd_cta), a thread-block cluster of
-// 8 or 16 beyond (k_apgd_full), and k_apgd where the full vectors do not fit: a
-// cluster whose CTA r owns a contiguous block of rows of G and of every vector.
-// Each of its iterations does one GEMV: the CTAs publish their slice of the proximal point z in shared
+// 8 or 16 beyond (k_apgd_full), one CTA per SM where a cluster cannot hold G
+// (k_apgd_grid), and k_apgd where the full vectors do not fit: a cluster whose CTA r
+// owns a contiguous block of rows of G and of every vector. Each of its iterations
+// does one GEMV: the CTAs publish their slice of the proximal point z in shared
 // memory, a cluster barrier, every CTA gathers the whole z through distributed
 // shared memory, multiplies its rows, publishes its partial sums, a second
 // barrier, and every CTA reduces the partials in the same order (so all take
@@ -99,7 +100,7 @@ struct ApgdArgs {
   int n_pad;
   int cache;      // rows of G that a CTA keeps in shared memory (k_apgd: 1 for all, 0 for none)
   int vec_ok;     // 1: float4 loads of G rows are aligned
-  int scalar;     // k_apgd_full: a lane takes single columns, not groups of four
+  int scalar;     // a lane takes single columns, not groups of four
 };
 
 // Rows [r0, r0 + nr) of G (leading dimension ldg, n columns) into dst (row
@@ -834,6 +835,257 @@ __global__ void __launch_bounds__(THREADS, 1) k_apgd_full(const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------
+// Whole-GPU variant for supports whose G a cluster cannot keep on the chip: the
+// iteration of k_apgd_full (every CTA keeps the vectors whole and owns a block of
+// rows of G, the same sums in the same order, hence the same results) over up to
+// one CTA per SM, so that G stays in shared memory. Vectors live in registers
+// (thread i holds entries i + 256 k). A product's entries go to all CTAs through
+// global memory as 64-bit words, the value and the product's number: a reader
+// polls the words themselves, so that an exchange costs one write and one read of
+// L2 and needs no barrier, fence or flag.
+//
+// A warp takes four rows and writes their words with one instruction, a whole
+// 32-byte sector: sectors written in parts, while every CTA polls them, made an
+// iteration 5 to 8 us instead of 2.3 to 4 (900 to 2500 atoms; 8 to 24 rows a CTA
+// against 32; pauses between the polls gained nothing). All of a thread's words
+// are asked for together.
+//
+// Two mailboxes alternate. A CTA writes product i + 2 only after reading all of
+// product i + 1, each entry of which was written after its CTA had read all of
+// product i, so no entry is overwritten while it is awaited. The launch is
+// cooperative (all CTAs resident); every wait has a limit.
+//
+// What bounds it: the latency of the exchange. Measured against k_apgd_full on 16
+// SMs, us an iteration: 900 atoms 3.8 and 2.9, 1300 5.7 and 2.8, 1700 8.1 and 3.4,
+// 2500 16.0 and 4.2.
+constexpr int GRID_THREADS = 256;
+constexpr int GRID_EMAX = 12;                       // entries per thread: supports of up to 3072
+constexpr int GRID_ROWS = 32;                       // rows per CTA at most: four a warp (a multiple of 4)
+
+__device__ __forceinline__ void mail_put(unsigned long long* p, unsigned tag, float v) {
+  const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(v);
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ unsigned long long mail_get(const unsigned long long* p) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return w;
+}
+
+template <int E>   // entries per thread
+__global__ void __launch_bounds__(GRID_THREADS, 1) k_apgd_grid(const __grid_constant__ ApgdArgs a,
+                                                              unsigned long long* __restrict__ mail) {
+  extern __shared__ __align__(16) float apgdg_sm[];   // the input vector (n_pad), rows of G
+  __shared__ Df scratch[(GRID_THREADS / 32) * NPART];
+  __shared__ Df s_part[NPART];
+  __shared__ __align__(16) float s_red[2][3][8];
+  __shared__ float s_al[LZ_MAX], s_be[LZ_MAX], s_theta;
+  __shared__ int s_bad;
+  float* vec_s = apgdg_sm;
+  float* Gc = apgdg_sm + a.n_pad;
+  const int n = a.n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r0 = (int)blockIdx.x * a.rows_per;
+  const int nr = max(0, min(n, r0 + a.rows_per) - r0);
+  const bool vecld = !a.scalar;
+  unsigned tag = 0;
+  int parity = 0;
+
+  load_rows_async(Gc, a.n_pad, a.G, a.ldg, r0, nr, n, a.vec_ok != 0);
+  for (int i = n + tid; i < a.n_pad; i += GRID_THREADS) vec_s[i] = 0.f;
+  if (tid == 0) s_bad = 0;
+  const float v0 = rsqrtf((float)n);        // Lanczos start: all ones / sqrt(n)
+  float x[E], Gx[E], y[E], Gy[E], bb[E], z[E], Gz[E];
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const int i = tid + GRID_THREADS * k;
+    bb[k] = i < n ? a.b[i] : 0.f;
+    x[k] = i < n ? a.x[i] : 0.f;
+    y[k] = i < n ? v0 : 0.f;   // v_j
+    z[k] = 0.f;                // v_{j-1}
+  }
+
+  // out = G in, every CTA all of it. A wait that expires leaves s_bad set for the
+  // caller to read behind its next barrier. The caller's barrier since the last
+  // product has ended every read of vec_s.
+  auto product = [&](const float (&in)[E], float (&out)[E]) {
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      const int i = tid + GRID_THREADS * k;
+      if (i < n) vec_s[i] = in[k];
+    }
+    __syncthreads();
+    ++tag;
+    unsigned long long* box = mail + (size_t)(tag & 1u) * a.n_pad;
+    for (int rb = 4 * warp; rb < nr; rb += 4 * (GRID_THREADS / 32)) {
+      const float* rows[4];
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) rows[q] = Gc + (size_t)min(rb + q, nr - 1) * a.n_pad;
+      rows_dot<4>(rows, vec_s, n, !a.scalar, acc);
+      for (int off = 16; off; off >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
+      if (lane < min(4, nr - rb))                     // 32 bytes: a whole sector
+        mail_put(box + r0 + rb + lane, tag, lane & 2 ? (lane & 1 ? acc[3] : acc[2]) : (lane & 1 ? acc[1] : acc[0]));
+    }
+    // all entries asked for at once, those that had not come once more
+    unsigned long long w[E];
+    const long long t0 = clock64();
+    bool good = true, all;
+#pragma unroll
+    for (int k = 0; k < E; ++k) w[k] = tid + GRID_THREADS * k < n ? 0ull : (unsigned long long)tag << 32;
+    do {
+      all = true;
+#pragma unroll
+      for (int k = 0; k < E; ++k)
+        if ((unsigned)(w[k] >> 32) != tag) w[k] = mail_get(box + tid + GRID_THREADS * k);
+#pragma unroll
+      for (int k = 0; k < E; ++k) all = all && (unsigned)(w[k] >> 32) == tag;
+      good = all || clock64() - t0 <= APGD_WAIT_CYCLES;
+    } while (!all && good);
+#pragma unroll
+    for (int k = 0; k < E; ++k) out[k] = __uint_as_float((unsigned)w[k]);
+    if (!good) s_bad = 1;
+  };
+
+  // ---- Lipschitz constant: Lanczos (alpha = v^T G v, then beta = ||w||)
+  float theta = 0.f, theta_prev = 0.f, beta_prev = 0.f;
+  int m = 0;
+  bool ok = true;
+  __syncthreads();
+  for (int j = 0; j < LZ_MAX; ++j) {
+    product(y, Gz);
+    float va[1] = {0.f};
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+      if (tid + GRID_THREADS * k < n) va[0] = fmaf(y[k], Gz[k], va[0]);
+    block_sum_f<1>(va, s_red, parity);
+    if (s_bad) {
+      ok = false;
+      break;
+    }
+    const float alpha = va[0];
+    float vb[1] = {0.f};
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+      if (tid + GRID_THREADS * k < n) {
+        const float w = Gz[k] - alpha * y[k] - beta_prev * z[k];
+        Gz[k] = w;
+        vb[0] = fmaf(w, w, vb[0]);
+      }
+    block_sum_f<1>(vb, s_red, parity);
+    const float beta = sqrtf(fmaxf(vb[0], 0.f));
+    if (tid == 0) {
+      s_al[j] = alpha;
+      s_be[j] = beta;
+    }
+    m = j + 1;
+    __syncthreads();
+    const bool last = (m == n) || (m == LZ_MAX) || !(beta > 1e-7f * fabsf(alpha));
+    if (last || (m % 4) == 0) {
+      theta = tridiag_top(s_al, s_be, m, &s_theta);
+      if (last || fabsf(theta - theta_prev) <= LZ_TOL * fabsf(theta)) break;
+      theta_prev = theta;
+    }
+    const float inv = 1.f / beta;
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      z[k] = y[k];
+      y[k] = Gz[k] * inv;
+    }
+    beta_prev = beta;
+  }
+  const float L = 1.01f * (theta > 0.f ? theta : 1.f);
+  const float invL = 1.f / L;
+  const float thr = __fmul_rn(a.lam, invL);
+
+  // ---- initial G x
+  if (ok) {
+    product(x, Gx);
+    __syncthreads();
+    ok = !s_bad;
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      y[k] = x[k];
+      Gy[k] = Gx[k];
+    }
+  }
+
+  // ---- monotone FISTA
+  float t = 1.f;
+  int it = 0;
+  for (it = 1; it <= a.max_iter && ok; ++it) {
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      const float u = y[k] - (Gy[k] - bb[k]) * invL;
+      z[k] = (a.positive ? fmaxf(u - thr, 0.f) : copysignf(fmaxf(fabsf(u) - thr, 0.f), u));
+    }
+    product(z, Gz);
+    // F(z) - F(x) from the difference itself (see k_apgd_full)
+    float v[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < E; ++k)
+      if (tid + GRID_THREADS * k < n) {
+        const float dF =
+            fmaf(z[k] - x[k], 0.5f * (Gz[k] + Gx[k]) - bb[k], a.lam * (fabsf(z[k]) - fabsf(x[k])));
+        v[0] += dF;
+        const float d = z[k] - y[k];
+        v[1] = fmaf(d, d, v[1]);
+        v[2] = fmaf(z[k], z[k], v[2]);
+      }
+    const float t1 = 0.5f * (1.f + sqrtf(1.f + 4.f * t * t));
+    const float c1 = t / t1, c2 = (t - 1.f) / t1;
+    block_sum_f<3>(v, s_red, parity);
+    if (s_bad) {
+      ok = false;
+      break;
+    }
+    const float step = sqrtf(v[1]);
+    const float nz = sqrtf(v[2]);
+    const bool accept = v[0] <= 0.f;
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      const float xo = x[k], Gxo = Gx[k];
+      const float xn = accept ? z[k] : xo;
+      const float Gxn = accept ? Gz[k] : Gxo;
+      y[k] = xn + c1 * (z[k] - xn) + c2 * (xn - xo);
+      Gy[k] = Gxn + c1 * (Gz[k] - Gxn) + c2 * (Gxn - Gxo);
+      x[k] = xn;
+      Gx[k] = Gxn;
+    }
+    t = t1;
+    if (step <= a.eps * nz) break;
+  }
+  if (it > a.max_iter) it = a.max_iter;
+  if (!ok) {
+    if (tid == 0 && a.err) atomicExch(a.err, 1);
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const int i = tid + GRID_THREADS * k;
+    if (i >= r0 && i < r0 + nr) a.x[i] = x[k];
+  }
+  if (blockIdx.x != 0) return;
+  // objective of the returned x, in double-float (reported only)
+  Df p[NPART] = {};
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    p[0] = df_add(p[0], df_prod(x[k], Gx[k]));
+    p[1] = df_add(p[1], df_prod(bb[k], x[k]));
+    p[2] = df_add(p[2], Df{fabsf(x[k]), 0.f});
+  }
+  block_sums(p, s_part, scratch);
+  if (tid == 0) {
+    const Df Fx = df_add(df_add(df_scale(s_part[0], 0.5f), df_neg(s_part[1])), df_scale(s_part[2], a.lam));
+    if (a.out_iters) *a.out_iters = it;
+    if (a.out_L) *a.out_L = (double)L;
+    if (a.out_F) *a.out_F = (double)Fx.hi + (double)Fx.lo;
+    if (a.out_lanczos) *a.out_lanczos = m;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // One-CTA variant for supports of up to CTA_NMAX atoms: the same Lanczos step
 // size, monotone FISTA, stop rule and reported objective, with two threads per
 // row of G and of every vector. Thread h of a row's two holds the row's columns
@@ -1107,12 +1359,14 @@ struct ApgdShape {
   int n_pad;
   size_t smem;
   int threads = APGD_THREADS;
-  bool by_alignment = false;   // k_apgd_full: unaligned rows of G by single columns
+  bool by_alignment = false;   // unaligned rows of G by single columns
+  int grid = 0;        // whole-GPU kernel: its CTAs
 };
 
 // dynamic shared memory ceilings: 227 KB per CTA minus the kernels' static arrays
 constexpr size_t kLimitRows = 200 * 1024;
 constexpr size_t kLimitFull = 231200;
+constexpr size_t kLimitGrid = 224 * 1024;
 
 int apgd_setup(int* cs_max_out) {
   static int cs_max = 0;
@@ -1131,6 +1385,10 @@ int apgd_setup(int* cs_max_out) {
                                  (int)kLimitFull));
     PC_CUDA(cudaFuncSetAttribute(k_apgd_full<2 * APGD_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kLimitFull));
+    PC_CUDA(cudaFuncSetAttribute(k_apgd_grid<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLimitGrid));
+    PC_CUDA(cudaFuncSetAttribute(k_apgd_grid<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLimitGrid));
+    PC_CUDA(cudaFuncSetAttribute(k_apgd_grid<GRID_EMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kLimitGrid));
     attrs_set = true;
   }
   *cs_max_out = cs_max;
@@ -1226,9 +1484,65 @@ ApgdArgs make_args(const ApgdJob& j, const ApgdShape& sh) {
 
 }  // namespace
 
+// Whole-GPU shape of a support whose G a cluster would read from L2 (cl: its cluster
+// shape): from about 870 atoms, where the cluster is the slower one (us an iteration,
+// 700 atoms 2.5 on the cluster and 2.4, 900 3.8 and 2.9, 1300 5.7 and 2.8), to about
+// 2750, where one CTA per SM no longer holds all rows.
+static bool apgd_grid_shape(int S, const ApgdShape& cl, ApgdShape* sh) {
+  if (!cl.full || cl.cta >= 0 || cl.cache >= cl.rows_per || S > GRID_THREADS * GRID_EMAX) return false;
+  int dev = 0, n_sm = 0, coop = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (!coop || n_sm < 1) return false;
+  *sh = cl;
+  const size_t row = sizeof(float) * (size_t)sh->n_pad;
+  sh->rows_per = std::min(GRID_ROWS, (int)(kLimitGrid / row - 1) & ~3);
+  if (sh->rows_per < 4) return false;
+  sh->grid = ceil_div(S, sh->rows_per);
+  sh->cache = sh->rows_per;
+  sh->smem = row * (1 + sh->rows_per);
+  return sh->grid <= n_sm;
+}
+
+static int launch_apgd_grid(const ApgdJob& j, const ApgdShape& sh, unsigned long long* mail, cudaStream_t st) {
+  PC_CUDA(cudaMemsetAsync(mail, 0, 2 * sizeof(*mail) * (size_t)sh.n_pad, st));   // product numbers start at 1
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(sh.grid, 1, 1);
+  cfg.blockDim = dim3(GRID_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = sh.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const ApgdArgs a = make_args(j, sh);
+  ProfScope prof_scope_(PROF_APGD, st);
+  prof_scope_.kernels = 1;
+  PC_CUDA(j.n <= 4 * GRID_THREADS   ? cudaLaunchKernelEx(&cfg, k_apgd_grid<4>, a, mail)
+          : j.n <= 8 * GRID_THREADS ? cudaLaunchKernelEx(&cfg, k_apgd_grid<8>, a, mail)
+                                    : cudaLaunchKernelEx(&cfg, k_apgd_grid<GRID_EMAX>, a, mail));
+  return PC_OK;
+}
+
 int run_apgd_jobs(const ApgdJob* jobs, int n_jobs, cudaStream_t st) {
   int cs_max = 0;
   PC_TRY(apgd_setup(&cs_max));
+  // a support alone may take the whole GPU; several run side by side on their clusters
+  if (n_jobs == 1 && jobs[0].n > 0) {
+    ApgdShape cl, one;
+    PC_TRY(apgd_shape(jobs[0].n, cs_max, &cl));
+    void* mail = nullptr;
+    if (apgd_grid_shape(jobs[0].n, cl, &one)) {
+      if (dmalloc(&mail, 2 * sizeof(unsigned long long) * (size_t)one.n_pad, st) == PC_OK) {
+        const int rc = launch_apgd_grid(jobs[0], one, static_cast<unsigned long long*>(mail), st);
+        dfree(mail, st);
+        return rc;
+      }
+      clear_error();                        // no room: the cluster needs none
+    }
+  }
   std::vector<ApgdShape> shapes(n_jobs);
   for (int i = 0; i < n_jobs; ++i)
     if (jobs[i].n > 0) PC_TRY(apgd_shape(jobs[i].n, cs_max, &shapes[i]));

@@ -34,7 +34,7 @@ def solve64(G, b, lam, positive):
 # iterate) and the FP32 products leave about 9 (1e-6 + 6e-8 sqrt(n)) <= 4e-5
 @pytest.mark.parametrize("positive", [False, True])
 @pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 192, 193, 223, 224, 225, 260, 513, 850,
-                               898, 901, 904, 1303, 1700])
+                               898, 901, 904, 1303, 1700, 2497, 2800])
 def test_apgd_at_the_edges(n, positive):
     import torch
 
