@@ -225,6 +225,9 @@ int launch_gram_thin(const int4* vis_fx, const float2* V, int64_t M, const float
 int launch_d2f(const double* in, int n, float* out, cudaStream_t st);
 int launch_gram_finalize_perm(const double* acc, int ldacc, int n_new, int n_act, const int32_t* perm,
                               float* G, int ldg, float* b, cudaStream_t st);
+int launch_make_atoms_flagged(const int32_t* idx, const float* x, int S, int N, double dl, float4* atoms, int* dflag,
+                              cudaStream_t st);
+int check_atoms_flag(int flag);
 int make_atoms_checked(const int32_t* idx, const float* x, int S, int N, double dl,
                        float4* atoms, int* dflag, cudaStream_t st);
 
@@ -303,6 +306,17 @@ struct Resample {
   int Nt = 0, G = 0;    // side of the transforms' image and of their grid
   double d = 1.0, beta = 0.0;
 };
+// A plan's device scalars (dscal, uscal, iscal: one block, so that one copy reads
+// them), and what a certificate reads back of them (pinned).
+struct Scalars {
+  double d[8];
+  unsigned u[8];
+  int32_t i[8];
+};
+struct Readback {
+  Scalars s;
+  int32_t bad_atoms;
+};
 struct BandTable {
   int* first = nullptr;
   float* w = nullptr;
@@ -340,6 +354,8 @@ struct pc_plan_s {
   double fov = 0, dl = 0, beta = 0;
   double w0 = 0, dw = 1, s_c = 0, w_min = 0, w_max = 0;
   bool wstack = false;
+  pc::Readback* readback = nullptr;       // pinned, and the event behind its index check (pc_certificate)
+  cudaEvent_t atoms_read = nullptr;
   pc::PhaseScale phase;   // fixed-point scales of the residual's w-term
   int grid_mode = 0;  // 0 auto, 1 CUDA cores, 2 tensor cores, 3 CUDA cores over plane
                       // windows (2 and 3: w-stacking only; else mode 1 runs)

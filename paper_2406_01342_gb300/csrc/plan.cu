@@ -890,9 +890,9 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   PC_TRY(dev_alloc_t(p, &p->mu, (size_t)NN));
   PC_TRY(dev_alloc_t(p, &p->mark, (size_t)NN));
   PC_CUDA(cudaMemsetAsync(p->mark, 0, NN, st));
-  PC_TRY(dev_alloc_t(p, &p->dscal, 8));
-  PC_TRY(dev_alloc_t(p, &p->uscal, 8));
-  PC_TRY(dev_alloc_t(p, &p->iscal, 8));
+  PC_TRY(dev_alloc_t(p, &p->dscal, sizeof(Scalars) / sizeof(double)));
+  p->uscal = reinterpret_cast<unsigned*>(p->dscal + 8);
+  p->iscal = reinterpret_cast<int32_t*>(p->uscal + 8);
   PC_CUDA(cudaMemsetAsync(p->iscal, 0, 8 * sizeof(int32_t), st));
   p->sel_blocks_n = ceil_div(NN, kSelItems);
   PC_TRY(dev_alloc_t(p, &p->sel_blocks, (size_t)p->sel_blocks_n + 2));
@@ -1173,6 +1173,8 @@ extern "C" void pc_plan_destroy(pc_plan_t p) {
   // (as cudaFree would), then return them to the pool
   cudaDeviceSynchronize();
   for (void* q : p->owned) dfree(q, 0);
+  if (p->readback) pinned_put(p->readback);
+  if (p->atoms_read) cudaEventDestroy(p->atoms_read);
   p->atomsA.release();
   p->atomsB.release();
   p->idxA.release();

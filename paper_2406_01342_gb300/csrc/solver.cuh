@@ -24,7 +24,7 @@ int adjoint_grid_impl(pc_plan_s* p, const float2* h, float* img, float scale, un
 int check_plan(pc_plan_s* p, const char* fn);
 int check_dev(const void* ptr, bool needed, const char* fn, const char* name);
 // synchronises st and reports an expired bounded wait of the tensor-core gridding
-int grid_flag_sync(pc_plan_s* p, cudaStream_t st, const char* fn);
+int grid_flag_sync(pc_plan_s* p, cudaStream_t st, const char* fn, Scalars* pinned = nullptr);
 float bits_to_float(unsigned b);
 float key_to_float(unsigned key);   // inverse of float_order_key (0 -> -infinity)
 

@@ -459,19 +459,29 @@ int launch_make_atoms(const int32_t* idx, const float* x, int S, int N, double d
   return PC_OK;
 }
 
-// Validating variant for the public entry points: returns PC_ERR_INVALID_ARG
-// when idx is not strictly ascending inside [0, N^2). Synchronises the stream.
-int make_atoms_checked(const int32_t* idx, const float* x, int S, int N, double dl,
-                       float4* atoms, int* dflag, cudaStream_t st) {
-  if (S <= 0) return PC_OK;
+// Validating variant for the public entry points: *dflag is set when idx is not
+// strictly ascending inside [0, N^2).
+int launch_make_atoms_flagged(const int32_t* idx, const float* x, int S, int N, double dl, float4* atoms, int* dflag,
+                              cudaStream_t st) {
   PC_CUDA(cudaMemsetAsync(dflag, 0, sizeof(int), st));
   k_make_atoms<<<ceil_div(S, 256), 256, 0, st>>>(idx, x, S, N, dl, atoms, dflag, nullptr);
   PC_LAUNCH_CHECK();
+  return PC_OK;
+}
+
+int check_atoms_flag(int flag) {
+  return flag ? fail(PC_ERR_INVALID_ARG, "support indices must be strictly ascending in [0, N*N)") : PC_OK;
+}
+
+// The same with the check read back: PC_ERR_INVALID_ARG. Synchronises the stream.
+int make_atoms_checked(const int32_t* idx, const float* x, int S, int N, double dl,
+                       float4* atoms, int* dflag, cudaStream_t st) {
+  if (S <= 0) return PC_OK;
+  PC_TRY(launch_make_atoms_flagged(idx, x, S, N, dl, atoms, dflag, st));
   int h = 0;
   PC_CUDA(cudaMemcpyAsync(&h, dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
   PC_CUDA(cudaStreamSynchronize(st));
-  if (h) return fail(PC_ERR_INVALID_ARG, "support indices must be strictly ascending in [0, N*N)");
-  return PC_OK;
+  return check_atoms_flag(h);
 }
 
 PhaseScale phase_scale(double w_max, double s_max) {
