@@ -21,7 +21,9 @@
 // consecutive output rows, whose bands overlap, so an input value is loaded once
 // for eight products; the weights come from a table of eight per input row
 // (zeros outside a band), broadcast from shared memory. What bounds it: those
-// shared-memory reads, three for eight products.
+// shared-memory reads, three for eight products, and on small images the latency of
+// the loads (a thread that summed four groups in turn left seven warps an SM; a
+// thread a group: both applications at 2048 x 2048 66 -> 38 us, at 1100 34 -> 21).
 #include <cmath>
 
 #include "pc_internal.cuh"
@@ -29,8 +31,9 @@
 namespace pc {
 namespace {
 
-constexpr int RS_COLS = 128;   // columns (threads) per CTA
+constexpr int RS_COLS = 128;   // columns per CTA
 constexpr int RS_ROWS = 32;    // output rows per CTA: four groups of eight
+constexpr int RS_THREADS = RS_COLS * (RS_ROWS / 8);   // a column and a group each
 
 constexpr int RS_TERMS = 96;   // most terms of the window's power series (beta <= 63)
 
@@ -103,24 +106,24 @@ __global__ void k_band_down(const __grid_constant__ Taps t, int groups, int widt
 // out[c][o] = scale * sum_t w[o][t] in[first + t][c]: in has n_in rows of n_cols,
 // out n_cols rows of n_out (transposed). The last application of the adjoint
 // also takes the maxima (maxbits, as the FFT epilogue).
-__global__ void __launch_bounds__(RS_COLS)
+__global__ void __launch_bounds__(RS_THREADS)
 k_band_apply(const float* __restrict__ in, int n_in, int n_cols, const int* __restrict__ first,
              const float* __restrict__ w, int width, float* __restrict__ out, int n_out, float scale,
              unsigned* __restrict__ maxbits) {
   extern __shared__ float4 rs_w[];                         // 4 groups x width x 8 weights
   __shared__ float tile[RS_ROWS][RS_COLS + 1];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, col = tid % RS_COLS, g = tid / RS_COLS;
   const int c0 = blockIdx.x * RS_COLS, o0 = blockIdx.y * RS_ROWS;
-  const int c = min(c0 + tid, n_cols - 1);
+  const int c = min(c0 + col, n_cols - 1);
   const int groups = (n_out + 7) / 8, g0 = o0 / 8, gn = min(RS_ROWS / 8, groups - g0);
   const float4* src = reinterpret_cast<const float4*>(w) + (size_t)g0 * width * 2;
-  for (int e = tid; e < gn * width * 2; e += RS_COLS) rs_w[e] = src[e];
+  for (int e = tid; e < gn * width * 2; e += RS_THREADS) rs_w[e] = src[e];
   __syncthreads();
-  for (int g = 0; g < gn; ++g) {
+  if (g < gn) {
     const int f = first[g0 + g];
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const float4* wg = rs_w + (size_t)g * width * 2;
-#pragma unroll 4
+#pragma unroll 8
     for (int t = 0; t < width; ++t) {
       const float v = in[(size_t)min(max(f + t, 0), n_in - 1) * n_cols + c];
       const float4 a = wg[2 * t], b = wg[2 * t + 1];
@@ -134,7 +137,7 @@ k_band_apply(const float* __restrict__ in, int n_in, int n_cols, const int* __re
       acc[7] = fmaf(b.w, v, acc[7]);
     }
 #pragma unroll
-    for (int r = 0; r < 8; ++r) tile[8 * g + r][tid] = acc[r] * scale;
+    for (int r = 0; r < 8; ++r) tile[8 * g + r][col] = acc[r] * scale;
   }
   __syncthreads();
   // 32 consecutive outputs of one column per warp
@@ -142,7 +145,7 @@ k_band_apply(const float* __restrict__ in, int n_in, int n_cols, const int* __re
   float amax = 0.f;
   unsigned skey = 0;   // order-preserving key of the signed maximum (0 below every number)
   if (o < n_out) {
-    for (int q = warp; q < RS_COLS && c0 + q < n_cols; q += RS_COLS / 32) {
+    for (int q = warp; q < RS_COLS && c0 + q < n_cols; q += RS_THREADS / 32) {
       const float m = tile[lane][q];
       out[(size_t)(c0 + q) * n_out + o] = m;
       amax = fmaxf(amax, fabsf(m));
@@ -170,7 +173,7 @@ int apply(const float* in, int n_in, int n_cols, const BandTable& t, float* out,
     PC_CUDA(cudaFuncSetAttribute(k_band_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
     attr = true;
   }
-  k_band_apply<<<dim3(ceil_div(n_cols, RS_COLS), ceil_div(n_out, RS_ROWS)), RS_COLS, smem, st>>>(
+  k_band_apply<<<dim3(ceil_div(n_cols, RS_COLS), ceil_div(n_out, RS_ROWS)), RS_THREADS, smem, st>>>(
       in, n_in, n_cols, t.first, t.w, t.width, out, n_out, scale, maxbits);
   PC_LAUNCH_CHECK();
   return PC_OK;
