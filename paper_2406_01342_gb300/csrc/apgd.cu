@@ -36,6 +36,7 @@
 
 #include <cmath>
 
+#include "apgd_rows.cuh"
 #include "lanczos.cuh"
 #include "pc_internal.cuh"
 
@@ -495,9 +496,9 @@ __device__ __forceinline__ void block_sum_f(float (&v)[K], float (*red)[3][8], i
 // complete).
 //
 // Two receive buffers alternate. A CTA sends product i + 2 into buffer i mod 2
-// only after it has received every CTA's product i + 1, which each CTA sends only
-// after it has consumed product i, so a buffer is never overwritten while it is
-// read. The mbarrier of a buffer is re-armed for product i + 2 before this CTA
+// only after it has received every CTA's product i + 1, which each CTA (all have
+// rows, see cluster_slice) sends only after it has consumed product i, so a buffer is
+// never overwritten while it is read. The mbarrier of a buffer is re-armed for product i + 2 before this CTA
 // sends product i + 1, and no phase can end twice while a thread still waits for
 // its first end: product i + 2 needs this CTA's own rows, which it sends after a
 // barrier of all its threads.
@@ -662,8 +663,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_apgd_full(const __grid_constant_
   const ApgdArgs& a = batch.job[blockIdx.x / cl.num_blocks()];
   const int rank = (int)cl.block_rank();
   const SmemF s = carve_full(apgdf_sm, a);
-  const int r0 = rank * a.rows_per;
-  const int nr = max(0, min(a.n, r0 + a.rows_per) - r0);
+  const RowSlice own = cluster_slice(a.n, (int)cl.num_blocks(), rank);
+  const int r0 = own.r0, nr = own.nr;
   const int n = a.n, tid = threadIdx.x, nt = APGD_THREADS;
   const int e0 = tid < nt ? tid : a.n_pad;    // first own entry of the vectors (none past the first threads)
   bool ok = true;
@@ -1399,7 +1400,7 @@ int apgd_shape(int S, int cs_max, ApgdShape* out) {
   const int n_pad = (S + 3) & ~3;
   // full-vector kernel: 2 receive buffers and 6 full vectors, and as many rows of
   // G as fit beside them; a CTA's rows are a multiple of 4 (16-byte stores)
-  auto rows_full = [&](int cs) { return (ceil_div(S, cs) + 3) & ~3; };
+  auto rows_full = [&](int cs) { return cluster_rows(S, cs); };
   const size_t vec_full = sizeof(float) * 8 * (size_t)n_pad, row_full = sizeof(float) * (size_t)n_pad;
   // row-slice kernel (larger supports): one full vector + 8 row slices
   auto bytes_rows = [&](int cs, bool cached) {
