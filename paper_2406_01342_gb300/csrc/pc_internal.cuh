@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "polyclean.h"
+#include "resample_rule.cuh"
 
 namespace pc {
 
@@ -300,12 +301,6 @@ int launch_fft_rows_big(pc_plan_s* p, cudaStream_t st);
 int launch_fft_cols_big(pc_plan_s* p, float* mu, float scale, unsigned* maxbits, cudaStream_t st);
 int launch_degrid_ffts_big(pc_plan_s* p, const float* img, cudaStream_t st);
 int make_xc_tensor_map(pc_plan_s* p);   // after xc is allocated
-// resample.cu: transforms on a smaller image of the same field
-struct Resample {
-  int K = 0;            // interpolation taps (0: the transforms run on the image itself)
-  int Nt = 0, G = 0;    // side of the transforms' image and of their grid
-  double d = 1.0, beta = 0.0;
-};
 // A plan's device scalars (dscal, uscal, iscal: one block, so that one copy reads
 // them), and what a certificate reads back of them (pinned).
 struct Scalars {
@@ -322,8 +317,7 @@ struct BandTable {
   float* w = nullptr;
   int width = 0;
 };
-Resample choose_resample(int N, int G, double turns);
-void resample_widths(const Resample& r, int N, int* up, int* down);
+// resample.cu: the interpolation between a plan's image and its smaller one
 int fill_band_tables(const Resample& r, int N, BandTable* up, BandTable* down, cudaStream_t st);
 int launch_upsample(pc_plan_s* p, float* img, float scale, unsigned* maxbits, cudaStream_t st);
 int launch_downsample(pc_plan_s* p, const float* img, cudaStream_t st);

@@ -752,9 +752,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
     // corner of the image; the transforms' smaller one reaches a little further
     const double half = 0.5 * N * p->dl, r2 = 2.0 * half * half;
     const double w_abs = std::max(std::fabs(p->w_min), std::fabs(p->w_max));
-    // turns per pixel: the baseline, and the slope |w| l / n of the w-term
-    const double turns = p->dl * (uv_max + w_abs * half / std::sqrt(1.0 - std::min(r2, 0.99)));
-    if (M > 0 && p->fft_warp != 0 && r2 < 0.4) p->resample = choose_resample(N, p->G_image, turns);
+    if (M > 0 && p->fft_warp != 0 && r2 < 0.4) p->resample = choose_resample(N, p->G_image, p->dl, uv_max, w_abs);
     if (p->resample.K > 0) {
       // its wider field takes more w-planes: not beyond the caller's cap
       const double h = 0.5 * p->resample.Nt * p->dl * p->resample.d, r2t = 2.0 * h * h;

@@ -11,9 +11,10 @@
 //   g(x) = sinc(x) I0(beta sqrt(1 - (2x/K)^2)) / I0(beta),  beta = pi K (1/2 - nu),
 //
 // the Kaiser-windowed sinc, for a band |frequency| <= nu cycles per small pixel
-// (nu from max |u|, |v| and the slope of the w-term over the field). With beta >=
-// 14.9, the rule below, it is within 1.5e-7 (rms 5e-8) of e^{2 pi i f x} over the
-// band: a twentieth of the operators' own error. The forward operator runs the
+// (nu from max |u|, |v| and the slope of the w-term, which climbs over the taps). With
+// beta >= 15.1, the rule's bound, it is within 1.5e-7 (rms 5e-8) of e^{2 pi i f x} over
+// the band and within 2.1e-7 of a wave whose frequency climbs: a tenth of the
+// operators' own error on the border. The forward operator runs the
 // transpose.
 //
 // Both directions are one kernel run twice: a banded matrix applied along the
@@ -24,8 +25,6 @@
 // shared-memory reads, three for eight products, and on small images the latency of
 // the loads (a thread that summed four groups in turn left seven warps an SM; a
 // thread a group: both applications at 2048 x 2048 66 -> 38 us, at 1100 34 -> 21).
-#include <cmath>
-
 #include "pc_internal.cuh"
 
 namespace pc {
@@ -34,28 +33,6 @@ namespace {
 constexpr int RS_COLS = 128;   // columns per CTA
 constexpr int RS_ROWS = 32;    // output rows per CTA: four groups of eight
 constexpr int RS_THREADS = RS_COLS * (RS_ROWS / 8);   // a column and a group each
-
-constexpr int RS_TERMS = 96;   // most terms of the window's power series (beta <= 63)
-
-// The window's series: I0(beta sqrt(y)) / I0(beta) = sum_k c[k] y^k, all terms
-// positive (c[k] = (beta / 2)^2k / k!^2 / I0(beta)).
-struct Taps {
-  double d;
-  int N, Nt, K, terms;
-  double c[RS_TERMS];
-};
-
-__host__ __device__ inline double tap_x(const Taps& t, int i) { return (i - t.N / 2) / t.d + t.Nt / 2; }
-__host__ __device__ inline int tap_first(const Taps& t, int i) { return (int)floor(tap_x(t, i)) - t.K / 2 + 1; }
-
-__device__ double tap_weight(const Taps& t, int i, int k) {
-  const double x = tap_x(t, i) - k, z = x * (2.0 / t.K), y = 1.0 - z * z;
-  if (!(y > 0.0)) return 0.0;
-  const double s = fabs(x) < 1e-9 ? 1.0 : sinpi(x) / (M_PI * x);
-  double w = 0.0;
-  for (int n = t.terms - 1; n >= 0; --n) w = fma(w, y, t.c[n]);
-  return s * w;
-}
 
 // Band tables: group g of eight output rows starts at input row first[g] and
 // holds `width` rows of eight weights. Up: output rows are the N pixels; down:
@@ -73,7 +50,8 @@ __global__ void k_band_up(const __grid_constant__ Taps t, int groups, int width,
   double v = 0.0;
   if (out < t.N && k >= 0 && k < t.Nt) {
     const int k0 = tap_first(t, out);
-    if (k >= k0 && k < k0 + t.K) v = tap_weight(t, out, k);
+    const double x = tap_x(t, out) - k;
+    if (k >= k0 && k < k0 + t.K) v = tap_weight(t, x, sinpi(x));
   }
   w[e] = (float)v;
 }
@@ -181,65 +159,8 @@ int apply(const float* in, int n_in, int n_cols, const BandTable& t, float* out,
 
 }  // namespace
 
-// The smallest grid of side 512 or more whose image of side G / 2 still samples
-// the visibilities: with K taps (16 .. 40) past the field's edge the pixels are d
-// = N / (G / 2 - K) wide, and K must reach beta = 14.9. The small grid oversamples
-// the pixels' field as much as the image's own grid does, up to 2.12: past that
-// the planes cost more than the accuracy gives (1100 x 1100 at 2.05 / 2.12 / 2.3:
-// errors 9.5e-7 / 6.7e-7 / 5.0e-7, against 7.2e-7 on the image's own grid; at 2.3 a
-// quarter more planes). turns: the most that a visibility turns per image pixel,
-// w-term included. Only grids of side 2048 and more are replaced: at 1024 the passes take 28 us of a 512 x 512 certificate's
-// 220, which the interpolation and a wider field's further w-planes would eat.
-Resample choose_resample(int N, int G, double turns) {
-  Resample r;
-  r.Nt = N;
-  r.G = G;
-  if (G < 2048) return r;
-  const double sigma = std::min(2.12, (double)G / N);
-  for (int g = 512; g < G; g *= 2)
-    for (int K = 16; K <= 40; K += 8) {
-      const double d = std::max((double)N / (g / 2 - K), sigma * N / g);
-      const double nu = turns * d, beta = M_PI * K * (0.5 - nu);
-      if (d < 1.0 || beta < 14.9) continue;
-      r.K = K;
-      r.Nt = g / 2;
-      r.G = g;
-      r.d = d;
-      r.beta = beta;
-      return r;
-    }
-  return r;
-}
-
-// Rows of the two tables: the widest band of eight output rows.
-void resample_widths(const Resample& r, int N, int* up, int* down) {
-  Taps t;
-  t.d = r.d;
-  t.N = N;
-  t.Nt = r.Nt;
-  t.K = r.K;
-  int wu = 0, wd = 0;
-  for (int i = 0; i < N; i += 8) wu = std::max(wu, tap_first(t, std::min(i + 7, N - 1)) + r.K - tap_first(t, i));
-  // an input pixel i meets rows [first, first + K): those of eight rows span at
-  // most (K + 7) d + 2 pixels
-  wd = (int)std::ceil((r.K + 7) * r.d) + 2;
-  *up = wu + 1;   // the device may round a pixel that falls on a small one the other way
-  *down = wd;
-}
-
 int fill_band_tables(const Resample& r, int N, BandTable* up, BandTable* down, cudaStream_t st) {
-  Taps t;
-  t.d = r.d;
-  t.N = N;
-  t.Nt = r.Nt;
-  t.K = r.K;
-  double i0 = 0.0, term = 1.0;
-  for (t.terms = 0; t.terms < RS_TERMS && (t.terms < 0.5 * r.beta || term > 1e-17 * i0); ++t.terms) {
-    t.c[t.terms] = term;
-    i0 += term;
-    term *= 0.25 * r.beta * r.beta / ((double)(t.terms + 1) * (t.terms + 1));
-  }
-  for (int k = 0; k < t.terms; ++k) t.c[k] /= i0;
+  const Taps t = make_taps(r, N);
   const int gu = ceil_div(N, 8), gd = ceil_div(r.Nt, 8);
   k_band_up<<<ceil_div((int64_t)gu * up->width * 8, 128), 128, 0, st>>>(t, gu, up->width, up->first, up->w);
   k_band_down<<<gd, 128, 0, st>>>(t, gd, down->width, up->first, up->w, up->width, down->first, down->w);
