@@ -145,10 +145,13 @@ k_band_apply(const float* __restrict__ in, int n_in, int n_cols, const int* __re
 
 int apply(const float* in, int n_in, int n_cols, const BandTable& t, float* out, int n_out, float scale,
           unsigned* maxbits, cudaStream_t st) {
-  const size_t smem = (size_t)(RS_ROWS / 8) * t.width * 8 * sizeof(float);
+  constexpr size_t row = (RS_ROWS / 8) * 8 * sizeof(float);   // of the table, four groups
+  if (t.width > RS_MAX_WIDTH) return fail(PC_ERR_CAPACITY, "interpolation: a band of %d rows", t.width);
+  const size_t smem = row * t.width;
   static bool attr = false;
   if (!attr) {
-    PC_CUDA(cudaFuncSetAttribute(k_band_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    PC_CUDA(cudaFuncSetAttribute(k_band_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(row * RS_MAX_WIDTH)));
     attr = true;
   }
   k_band_apply<<<dim3(ceil_div(n_cols, RS_COLS), ceil_div(n_out, RS_ROWS)), RS_THREADS, smem, st>>>(

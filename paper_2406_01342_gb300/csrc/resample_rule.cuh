@@ -97,7 +97,10 @@ inline Resample choose_resample(int N, int G, double dl, double uv_max, double w
   return r;
 }
 
-// Rows of the two tables: the widest band of eight output rows.
+// Rows of the two tables: the widest band of eight output rows. The kernel that applies
+// them has shared memory for RS_MAX_WIDTH rows (894 at 4096 x 4096 with 40 taps on a grid
+// of 512: (40 + 7) 4096 / 216 + 2).
+constexpr int RS_MAX_WIDTH = 896;
 inline void resample_widths(const Resample& r, int N, int* up, int* down) {
   Taps t;
   t.d = r.d;

@@ -1,7 +1,8 @@
 // Host-side check of the smaller image that the rule chooses (resample_rule.cuh): a
 // visibility's response on the smaller image, interpolated with the rule's taps,
 // against its value at the N x N image's border and at pixels inside, in float64, for
-// w-terms of none to nearly all of the turns and both signs.
+// w-terms of none to nearly all of the turns and both signs. And the rows of its
+// tables, over all sides and turns, against what the kernel has room for.
 // Prints "ok" and exits 0, or the failures and exits 1.
 #include "resample_rule.cuh"
 
@@ -68,6 +69,21 @@ int main() {
             bad = 1;
           }
         }
+  }
+  for (int N = 514; N <= 4096; N += 2) {
+    int G = 2048;
+    while (G < 2 * N) G *= 2;
+    for (int e = 0; e <= 4000; ++e) {
+      const double turns = 0.5 * e / 4000.0, dl = 0.05 / N;
+      const Resample r = choose_resample(N, G, dl, turns / dl, 0.0);
+      if (r.K == 0) continue;
+      int up, down;
+      resample_widths(r, N, &up, &down);
+      if (up > RS_MAX_WIDTH || down > RS_MAX_WIDTH) {
+        std::printf("N %d, %g turns: tables of %d and %d rows\n", N, turns, up, down);
+        return 1;
+      }
+    }
   }
   if (!bad) std::printf("ok\n");
   return bad;
