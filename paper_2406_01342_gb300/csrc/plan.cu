@@ -394,11 +394,16 @@ __global__ void k_pix_tab(PixGeom g, const double* __restrict__ rpsi, const doub
   const int b = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
   if (b > g.N / 2) return;
   const double l = a * g.dl, m = b * g.dl;
-  const double q = 1.0 - (l * l + m * m);
-  // 1 / n = q^(-1/2): an FP32 value and one Newton step (1e-13 relative)
+  const double r2 = l * l + m * m, q = 1.0 - r2;
+  // 1 / n = q^(-1/2) and 1 / (1 + n): an FP32 value and one Newton step each (1e-13
+  // relative). n - 1 = -r2 / (1 + n) keeps that accuracy; the difference q / n - 1 was off
+  // by 5e-14, which |w| multiplies into turns
   double rn = (double)rsqrtf((float)q);
   rn *= fma(-0.5 * q * rn, rn, 1.5);
-  const double s = q * rn - 1.0;     // n - 1
+  const double n1 = fma(q, rn, 1.0);
+  double rn1 = (double)(1.f / (float)n1);
+  rn1 *= fma(-n1, rn1, 2.0);
+  const double s = -r2 * rn1;        // n - 1
   double t = 0.0, rw = 1.0;
   if (g.wstack) {
     t = g.dw * (s - g.s_c);
