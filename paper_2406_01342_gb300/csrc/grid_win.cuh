@@ -44,6 +44,23 @@ __host__ __device__ __forceinline__ int4 chunk_after(const int2* wr, int Pw, int
   return make_int4(-1, 0, 1, 0);
 }
 
+// Slots of a CTA at most: a heavier tile is split into parts. Where the tiles alone are
+// eight CTAs an SM, a split costs more (adds to the grid instead of stores) than it
+// balances: `many`. With fewer, a CTA's share is what two CTAs on every SM would take,
+// up to 4096 slots: on the small grids of resampled plans (a few hundred tiles, the
+// middle ones heavy) the longest tile is otherwise the time. Gridding / degridding, us,
+// parts of 4096 (8192) slots and these: 540 x 540, 97k visibilities, 0.1 turns a pixel
+// 329 / 162 and 83 / 40, 0.2 turns 157 / 80 and 77 / 42; 960 x 960, 250k 317 / 157 and
+// 152 / 72; 1400 x 1400, 400k 190 / 119 and 168 / 118; 4096 slots are near the best from
+// 700k on. At least 16 slots a plane, since every part passes all planes of its tile
+// (1100 x 1100, 30k, 23 planes: 65 in parts of 4096, 73 of 256, 78 of 140).
+__host__ __device__ __forceinline__ int part_slots(long long slots, int tiles, int planes, int n_sm, int many) {
+  if (tiles >= 8 * n_sm) return many;
+  const long long share = (slots + 2 * n_sm - 1) / (2 * n_sm);
+  const int least = planes < 256 ? 16 * planes : 4096;
+  return (int)(share < least ? least : share > 4096 ? 4096 : share);
+}
+
 // Part `part` of `parts` of the slot range [bs, be): {first, count}; the
 // parts are contiguous and cover the range once.
 __host__ __device__ __forceinline__ int2 part_range(int bs, int be, int part, int parts) {

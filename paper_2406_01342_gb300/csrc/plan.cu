@@ -20,6 +20,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "grid_win.cuh"
 #include "pc_internal.cuh"
 
 namespace pc {
@@ -619,7 +620,7 @@ static int autotune(pc_plan_s* p, cudaStream_t st) {
     p->grid_mode = mode;
     const bool win = grid_win_mode(p);
     // window gridding: slots per CTA before a tile is split; else the sub-problem size
-    const std::vector<int> pieces = win ? std::vector<int>{1024, 4096, 16384, 65536}
+    const std::vector<int> pieces = win ? std::vector<int>{p->win_cap, 1024, 4096, 16384, 65536}
                                         : std::vector<int>{256, 512, 1024, 2048, 4096};
     for (int piece : pieces) {
       p->grid_mode = mode;
@@ -692,7 +693,7 @@ static int autotune(pc_plan_s* p, cudaStream_t st) {
   if (grid_win_mode(p)) {
     double best_dw = 1e300;
     int best_cap = p->dwin_cap;
-    for (int cap : {2048, 4096, 8192, 16384}) {
+    for (int cap : {p->dwin_cap, 2048, 4096, 8192, 16384}) {
       PC_TRY(split_dwsubs(p, cap, up));
       double us = 0.0;
       PC_TRY(time_us(st, 3, [&] { return launch_degrid_win(p, p->resid, st); }, &us));
@@ -1011,10 +1012,7 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   PC_TRY(dev_alloc_t(p, &p->subs, (size_t)p->sub_cap));
   PC_TRY(split_subs(p, piece, up));
   // window gridding: the bin offsets on the device, the tiles that hold slots,
-  // and the CTA list. Measured (2048^2 / 2M and 4096^2 / 10M): splitting a
-  // tile costs more than it balances once the tiles alone give eight CTAs per
-  // SM, so then only tiles beyond 65536 slots are split; with fewer tiles,
-  // parts of at most 4096 slots
+  // and the CTA list (gwin::part_slots)
   PC_TRY(dev_alloc_t(p, &p->win_off, (size_t)nbins + 1));
   PC_CUDA(cudaMemcpyAsync(p->win_off, off, sizeof(int) * ((size_t)nbins + 1), cudaMemcpyDeviceToDevice, st));
   p->win_tiles.clear();
@@ -1024,11 +1022,12 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   }
   p->wsub_cap = p->n_slots / 64 + (int64_t)p->win_tiles.size() + 1;
   PC_TRY(dev_alloc_t(p, &p->wsubs, (size_t)p->wsub_cap));
-  PC_TRY(split_wsubs(p, (int64_t)p->win_tiles.size() >= 8ll * n_sm ? 65536 : 4096, up));
+  const int n_tiles = (int)p->win_tiles.size();
+  PC_TRY(split_wsubs(p, gwin::part_slots(p->n_slots, n_tiles, p->P, n_sm, 65536), up));
   PC_TRY(dev_alloc_t(p, &p->dwsubs, (size_t)p->wsub_cap));
-  // window degridding: parts of at most 8192 slots (measured best or within
-  // 2 % of the best cap on 2048^2 / 2M and 4096^2 / 10M; the tuner times it)
-  PC_TRY(split_dwsubs(p, 8192, up));
+  // window degridding: no part writes the grid, so 8192 also with many tiles (measured
+  // best or within 2 % of the best on 2048^2 / 2M and 4096^2 / 10M; the tuner times it)
+  PC_TRY(split_dwsubs(p, gwin::part_slots(p->n_slots, n_tiles, p->P, n_sm, 8192), up));
   // grid rows that any visibility can reach: the rows of tile rows with a sub-problem
   {
     std::vector<char> row_on(p->nT, 0);
