@@ -359,8 +359,8 @@ int forward_grid_impl(pc_plan_s* p, const float* img, float2* y, cudaStream_t st
   if (grid_win_mode(p)) {
     PC_TRY(launch_degrid_win(p, y, st));
   } else {
-    if (p->T != DG_T || p->Qg > 8) return fail(PC_ERR_INVALID_ARG, "forward: needs 32-cell tiles, <= 8 planes");
-    const size_t smem = sizeof(float2) * (size_t)p->Qg * DG_T * DG_TP;
+    if (p->T != DG_T || p->Qd > 8) return fail(PC_ERR_INVALID_ARG, "forward: needs 32-cell tiles, <= 8 planes");
+    const size_t smem = sizeof(float2) * (size_t)p->Qd * DG_T * DG_TP;
     const float beta = (float)p->beta;
 #define PC_DEGRID_CASE(WW)                                                                              \
   case WW: {                                                                                            \
@@ -370,8 +370,8 @@ int forward_grid_impl(pc_plan_s* p, const float* img, float2* y, cudaStream_t st
                                    (int)(sizeof(float2) * 8 * DG_T * DG_TP)));                         \
       attr = true;                                                                                      \
     }                                                                                                   \
-    k_degrid<WW><<<p->n_sub, 256, smem, st>>>(p->subs, p->slot_vis, p->slot_geom, p->grid, G, p->nT, p->P, \
-                                              p->Qg, beta, ws, y);                                      \
+    k_degrid<WW><<<p->n_dsub, 256, smem, st>>>(p->dsubs, p->slot_vis, p->slot_geom, p->grid, G, p->nT,  \
+                                               p->P, p->Qd, beta, ws, y);                               \
     break;                                                                                              \
   }
     switch (p->W) {

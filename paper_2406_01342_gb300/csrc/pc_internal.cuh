@@ -379,6 +379,8 @@ struct pc_plan_s {
   int2* slot_vis = nullptr;      // {visibility, (a0 + 64) | (b0 + 64) << 8 | plane_start << 16}
   float4* slot_geom = nullptr;   // {gu - a0, gv - b0, xw - plane_start, tau (turns)}
   int4* subs = nullptr;          // gridding sub-problems {tile, plane group, start, end}
+  int4* dsubs = nullptr;         // the same of the degridding over plane groups
+  int n_dsub = 0, Qd = 0;        // their number, and planes per group
   int* win_off = nullptr;        // first slot of each (tile, plane pair) bin (nT^2 Pw + 1)
   int4* wsubs = nullptr;         // window gridding CTAs {tile, part, parts, slots}, heaviest first
   int4* dwsubs = nullptr;        // window degridding CTAs (the same form, their own split)

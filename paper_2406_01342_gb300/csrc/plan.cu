@@ -969,28 +969,32 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   // even waves of two CTAs per SM -- a few long sub-problems left over for a
   // second wave would otherwise double the gridding time.
   const int kMaxSlotsPerSub = 512;   // the autotuner's usual pick (smaller pieces: more CTAs in flight)
-  std::vector<int4> ranges;
-  int64_t total_slots = 0;
-  const int ngroups = ceil_div(p->P, p->Qg);
-  for (int t = 0; t < p->nT * p->nT; ++t) {
-    for (int gq = 0; gq < ngroups; ++gq) {
-      int q0 = gq * p->Qg;
-      // plane starts whose footprint meets the group, widened to whole pairs
-      // (the extra slots' footprints miss the group: zero weights there)
-      int ps_lo = 0, ps_hi = 0;
-      if (p->wstack) {
-        ps_lo = std::max(0, q0 - p->W + 1);
-        ps_hi = std::min(p->P - p->W, q0 + p->Qg - 1);
-      }
-      if (ps_hi < ps_lo) continue;
-      int s0 = hoff[(size_t)t * p->Pw + (ps_lo >> 1)];
-      int s1 = hoff[(size_t)t * p->Pw + (ps_hi >> 1) + 1];
-      if (s1 > s0) {
-        ranges.push_back(make_int4(t, gq, s0, s1));
-        total_slots += s1 - s0;
+  // the slot range of each (tile, group of Q planes) that holds any; returns the slots
+  auto plane_groups = [&](int Q, std::vector<int4>& out) {
+    int64_t total = 0;
+    for (int t = 0; t < p->nT * p->nT; ++t) {
+      for (int gq = 0; gq < ceil_div(p->P, Q); ++gq) {
+        int q0 = gq * Q;
+        // plane starts whose footprint meets the group, widened to whole pairs
+        // (the extra slots' footprints miss the group: zero weights there)
+        int ps_lo = 0, ps_hi = 0;
+        if (p->wstack) {
+          ps_lo = std::max(0, q0 - p->W + 1);
+          ps_hi = std::min(p->P - p->W, q0 + Q - 1);
+        }
+        if (ps_hi < ps_lo) continue;
+        int s0 = hoff[(size_t)t * p->Pw + (ps_lo >> 1)];
+        int s1 = hoff[(size_t)t * p->Pw + (ps_hi >> 1) + 1];
+        if (s1 > s0) {
+          out.push_back(make_int4(t, gq, s0, s1));
+          total += s1 - s0;
+        }
       }
     }
-  }
+    return total;
+  };
+  std::vector<int4> ranges;
+  const int64_t total_slots = plane_groups(p->Qg, ranges);
   int n_sm = 152;
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
   const int64_t want = 4ll * n_sm;
@@ -1011,6 +1015,26 @@ static int build_plan(pc_plan_s* p, const double* uvw, cudaStream_t st, int max_
   p->sub_cap = (int)(total_slots / stage + (int64_t)ranges.size() + 1);
   PC_TRY(dev_alloc_t(p, &p->subs, (size_t)p->sub_cap));
   PC_TRY(split_subs(p, piece, up));
+  // degridding over plane groups: its own groups and pieces. Its time is a thread's slots
+  // one after the other, Qd planes each, and eight planes of a tile leave room for three
+  // CTAs an SM: half the planes, or four beyond twelve. Pieces of whole passes of its 256
+  // threads (in the gridding's 320 the second pass was nearly empty), 512 slots where
+  // they still make five CTAs an SM. us, the gridding's groups and pieces and these: 512 x
+  // 512, 200k visibilities, 8 planes 60 and 49, 11 planes 55 and 55, 15 planes 64 and 56;
+  // 306 x 306, 118k, 8 planes 47 and 38; 400 x 400, 60k, 8 planes 35 and 29
+  if (!grid_win_mode(p) || p->want_tune) {
+    std::vector<int4> dr, ds;
+    p->Qd = !p->wstack ? 1 : p->P <= 12 ? ceil_div(p->P, 2) : 4;
+    const int64_t share = (plane_groups(p->Qd, dr) + want - 1) / want;
+    const int dpiece = share >= 3 * 256 ? 512 : share > 192 ? 256 : share > 128 ? 192 : 128;
+    for (const int4& r : dr) {
+      const int n = ceil_div(r.w - r.z, dpiece), sz = ceil_div(r.w - r.z, n);
+      for (int a = r.z; a < r.w; a += sz) ds.push_back(make_int4(r.x, r.y, a, std::min(r.w, a + sz)));
+    }
+    p->n_dsub = (int)ds.size();
+    PC_TRY(dev_alloc_t(p, &p->dsubs, std::max<size_t>(ds.size(), 1)));
+    PC_TRY(up.upload(p->dsubs, ds.data(), sizeof(int4) * ds.size()));
+  }
   // window gridding: the bin offsets on the device, the tiles that hold slots,
   // and the CTA list (gwin::part_slots)
   PC_TRY(dev_alloc_t(p, &p->win_off, (size_t)nbins + 1));
