@@ -8,9 +8,10 @@
 //   Gram        G = Re(Phi_S^H Phi_S),  b = Re(Phi_S^H V)
 //
 // Phases are generated on the fly: the lattice part i' U_k + j' V_k in exact
-// 32-bit fixed-point turns, the w-term as a double-float product, one FP32
-// sincospi per (visibility, atom) pair.
+// 32-bit fixed-point turns, the w-term as a double-float product or, in the residual,
+// as one of 32-bit integers (k_residual).
 #include <cmath>
+#include <type_traits>
 
 #include "pc_internal.cuh"
 
@@ -36,20 +37,52 @@ __device__ __forceinline__ int fixed32(float hi, float lo, float scale) {
   return __float2int_rn(hi * scale) + __float2int_rn(lo * scale);
 }
 
+// x e^{j theta} of a phase in 32-bit fixed-point turns: {x, sin, cos}.
+//  HALF   th holds a quarter turn more. Its top bit is the sign of a half turn, taken
+//         onto the weight; the next 23 become the mantissa of a float in [1, 2), that is
+//         an angle in [-pi/2, pi/2] to 2^-25 turns, where the fast sine and cosine are
+//         accurate to 4e-7
+//  FINE   the same with the last 8 bits added to the angle
+//  SLOW   sine and cosine of the phase itself, to the last bits of FP32
+enum PhaseKind { HALF, FINE, SLOW };
+template <PhaseKind KIND>
+__device__ __forceinline__ float3 weigh(unsigned th, int weight) {
+  float sn, cs;
+  if (KIND == SLOW) {
+    sincospif((float)(int)th * 4.656612873077393e-10f, &sn, &cs);   // 2^-31
+    return make_float3(__int_as_float(weight), sn, cs);
+  }
+  const float f = __uint_as_float(((th >> 8) & 0x7fffffu) | 0x3f800000u);
+  if (KIND == FINE) {
+    const float low = __uint_as_float((th & 0xffu) | 0x4b000000u);  // 2^23 + the last bits
+    __sincosf(fmaf(low, 1.46291807926716e-9f, fmaf(f, 3.14159265358979f, -4.72466082668777f)), &sn, &cs);
+  } else {
+    __sincosf(fmaf(f, 3.14159265358979f, -4.71238898038469f), &sn, &cs);
+  }
+  return make_float3(__int_as_float(weight ^ (int)(th & 0x80000000u)), sn, cs);
+}
+
+// Which kind: the error of a sum of few atoms is that of its phases, of many that of
+// the FP32 sums (relative error against 64 bits, the double-float kernel of before /
+// HALF / FINE / SLOW: 5 atoms x 10k visibilities 1.83e-7 / 2.13e-7 / 1.86e-7 / 0.79e-7, 10
+// x 200k 2.4e-7 / 2.6e-7 / 2.4e-7 / 1.7e-7, 120 x 1.2M 3.1e-7 / 3.1e-7 / 3.0e-7 /
+// 2.5e-7, 300 x 20k 3.9e-7 / 2.4e-7 / 2.1e-7 / 1.4e-7). Each kind is taken where it is
+// no further off than that kernel: HALF from 257 atoms, FINE (12 % slower) below, SLOW
+// (twice) for the few of which launch and visibilities are the time.
+constexpr int RES_SLOW_MAX = 16, RES_FINE_MAX = 256;
+constexpr int64_t RES_SLOW_M = 100000;
+
 // out = V - Phi_S x  (or Phi_S x when V is null); sumsq += ||out||^2 in float64.
 //
 // The phase i' U + j' V + w s of a (visibility, atom) pair stays in 32-bit
 // fixed-point turns: w and s = n - 1 are 32-bit integers at power-of-two scales
 // (PhaseScale), the 64-bit product is shifted to turns, and the sum wraps, which
-// is the exact reduction. Its top bit is the sign of a half turn, taken onto the
-// weight; the next 23 become the mantissa of a float in [1, 2), that is an angle
-// in [-pi/2, pi/2] to 2^-25 turns, where the fast sine and cosine are accurate to
-// 4e-7.
+// is the exact reduction.
 //
 // What bounds it: the two MUFU operations a phase, 16 a cycle and SM, so 8
 // phases a cycle. The double-float w-term with two roundings to the nearest turn
 // and an integer conversion (which shares that pipe) issued 24 instructions and
-// ran 4.1 phases a cycle; this is 12 instructions, none of them a conversion.
+// ran 4.1 phases a cycle; HALF is 12 instructions, FINE 14, none of them a conversion.
 //
 // A block's eight warps hold GROUPS groups, each summing its share of the atoms
 // for the same 256 / GROUPS x VPT visibilities, so that few visibilities still
@@ -77,8 +110,9 @@ k_residual(const int4* __restrict__ vis, const float2* __restrict__ V, int64_t M
     w[j] = fixed32(__int_as_float(q.z), __int_as_float(q.w), sc.w_scale);
     ar[j] = ai[j] = 0.f;
   }
+  const PhaseKind kind = S <= RES_SLOW_MAX && M < RES_SLOW_M ? SLOW : S <= RES_FINE_MAX ? FINE : HALF;
   // a quarter turn, so that the top bit tells the half, and the rounding of the shift by 8
-  const long long bias = (long long)(0x40000000u + 128u) << sc.shift;
+  const long long bias = (long long)(kind == SLOW ? 0u : kind == FINE ? 0x40000000u : 0x40000000u + 128u) << sc.shift;
   for (int s0 = 0; s0 < S; s0 += RES_CHUNK) {
     const int cnt = min(RES_CHUNK, S - s0);
     for (int t = tid; t < cnt; t += 256) {
@@ -88,22 +122,27 @@ k_residual(const int4* __restrict__ vis, const float2* __restrict__ V, int64_t M
                         __float_as_int(at.w));
     }
     __syncthreads();
+    auto sum = [&](auto k) {
 #pragma unroll 2
-    for (int t = group; t < cnt; t += GROUPS) {
-      const int4 at = sa[t];
+      for (int t = group; t < cnt; t += GROUPS) {
+        const int4 at = sa[t];
 #pragma unroll
-      for (int j = 0; j < VPT; ++j) {
-        const long long ws = (long long)w[j] * at.z + bias;
-        const unsigned th = (unsigned)at.x * (unsigned)u[j] + ((unsigned)at.y * (unsigned)v[j] +
-                            __funnelshift_r((unsigned)ws, (unsigned)((unsigned long long)ws >> 32), sc.shift));
-        const float f = __uint_as_float(((th >> 8) & 0x7fffffu) | 0x3f800000u);
-        const float x = __int_as_float(at.w ^ (int)(th & 0x80000000u));
-        float sn, cs;
-        __sincosf(fmaf(f, 3.14159265358979f, -4.71238898038469f), &sn, &cs);
-        ar[j] = fmaf(x, cs, ar[j]);
-        ai[j] = fmaf(-x, sn, ai[j]);
+        for (int j = 0; j < VPT; ++j) {
+          const long long ws = (long long)w[j] * at.z + bias;
+          const unsigned th = (unsigned)at.x * (unsigned)u[j] + ((unsigned)at.y * (unsigned)v[j] +
+                              __funnelshift_r((unsigned)ws, (unsigned)((unsigned long long)ws >> 32), sc.shift));
+          const float3 e = weigh<decltype(k)::value>(th, at.w);
+          ar[j] = fmaf(e.x, e.z, ar[j]);
+          ai[j] = fmaf(-e.x, e.y, ai[j]);
+        }
       }
-    }
+    };
+    if (kind == SLOW)
+      sum(std::integral_constant<PhaseKind, SLOW>());
+    else if (kind == FINE)
+      sum(std::integral_constant<PhaseKind, FINE>());
+    else
+      sum(std::integral_constant<PhaseKind, HALF>());
     __syncthreads();
   }
   if (GROUPS > 1) {
@@ -498,9 +537,11 @@ PhaseScale phase_scale(double w_max, double s_max) {
 }
 
 // The fixed-point kernel wherever the w-term stays within 32 turns (its 32-bit
-// factors then leave it 1.5e-8 turns; the configurations have 0.2 to 4), else the
-// double-float one. Visibilities per block by their number, so that there are two
-// blocks or more an SM (200k visibilities x 200 atoms: 44 us in blocks of 512).
+// factors then leave it 2e-8 turns rms, 6e-8 at most; the configurations have 0.2 to 4),
+// else the double-float one. Visibilities per block by their number, so that there are two
+// blocks or more an SM (200k visibilities x 200 atoms: 44 us in blocks of 512); for a
+// handful of atoms one a thread (8 atoms x 1.2M visibilities: 19.7 us with four a thread,
+// 17.3 with one).
 int launch_residual(const int4* vis_fx, const float2* V, int64_t M, const float4* atoms, int S,
                     float2* out, double* sumsq, const PhaseScale& sc, cudaStream_t st, const int32_t* S_dev) {
   ProfScope prof_scope_(PROF_RESIDUAL, st);
@@ -511,6 +552,8 @@ int launch_residual(const int4* vis_fx, const float2* V, int64_t M, const float4
                                                                            S_dev, sc)
   if (!sc.fixed)
     k_residual_wide<<<ceil_div(M, 256), 256, 0, st>>>(vis_fx, V, M, atoms, S, out, sumsq, S_dev);
+  else if (S <= RES_SLOW_MAX)
+    PC_RESIDUAL(1, 1);
   else if (M >= 1000000)
     PC_RESIDUAL(4, 1);
   else if (M >= 400000)
