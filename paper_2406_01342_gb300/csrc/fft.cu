@@ -399,10 +399,15 @@ static int cols_epilogue(pc_plan_s* p, float* mu, float scale, unsigned* maxbits
   if (fft_cols_warp(p)) {
     // warps per image row, a power of 2 <= P: the least planes one after the other in
     // whole waves of two CTAs on each of 152 SMs (nine planes on eight warps take two
-    // rounds, the second with one warp at work)
+    // rounds, the second with one warp at work); a sixteenth of a wave more counts for
+    // nothing. us of the pass with eight warps a row and with four: 306 rows and 10 planes
+    // 28.8 and 30.5, 340 35.5 and 32.9, 400 39.5 and 35.9, 512 47.2 and 37.5, 512 and 14
+    // planes 49.0 and 46.8; 256 and 10 planes 10.0 and 12.1, 512 and 8 18.4 and 29.0
+    constexpr int wave = 2 * 152;
     int wpr = 1, best = INT_MAX;
     for (int w = 8; w >= 1; w >>= 1) {
-      const int t = ceil_div(ceil_div(p->Nt, 8 / w), 2 * 152) * ceil_div(p->P, w);
+      const int ctas = ceil_div(p->Nt, 8 / w);
+      const int t = ceil_div(std::max(ctas - wave / 16, 1), wave) * ceil_div(p->P, w);
       if (w <= p->P && t < best) {
         best = t;
         wpr = w;
