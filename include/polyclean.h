@@ -65,8 +65,8 @@ typedef struct {
   int32_t kernel_width;   /* ES kernel width W in grid cells (default 7; 4..8)         */
   int32_t tile;           /* gridding tile side in cells (32, the only supported value) */
   int32_t max_planes;     /* cap on the number of w-planes (default 256)                */
-  int32_t grid_mode;      /* gridding: 0 (default) when w-stacking, mode 3 on grids of side
-                             >= 2048 (kernel_width <= 7), else tensor cores; CUDA cores
+  int32_t grid_mode;      /* gridding: 0 (default) when w-stacking, mode 3 for images with grids
+                             of side >= 2048 (kernel_width <= 7), else tensor cores; CUDA cores
                              without w-stacking. 1: FP32 CUDA cores; 2: tensor cores
                              whenever w-stacking; 3: FP32 CUDA cores over plane windows,
                              one CTA per tile, when w-stacking with kernel_width <= 7
@@ -187,10 +187,16 @@ int pc_plan(const double* uvw_dev, int64_t M, int32_t N, double fov_rad, const p
             void* stream, pc_plan_t* plan_out);
 void pc_plan_destroy(pc_plan_t plan);
 
-/* Plan geometry: oversampled grid side, tile side, number of w-planes, number
- * of binned (replicated) visibility slots, kernel width. Any pointer may be NULL. */
+/* Plan geometry: oversampled grid side of the N x N image, tile side, number of w-planes,
+ * number of binned (replicated) visibility slots, kernel width. Any pointer may be NULL.
+ * The w-planes' own grid may be smaller: pc_plan_transforms. */
 int pc_plan_info(pc_plan_t plan, int32_t* grid_side, int32_t* tile, int32_t* n_planes,
                  int64_t* n_slots, int32_t* kernel_width, double* dw);
+/* Grid and image that the w-planes are transformed on. grid_side is that of pc_plan_info
+ * and image_side is N, unless the visibilities do not resolve the pixels: then the
+ * planes are on a smaller grid, their image of the same field has image_side = grid_side
+ * / 2, and it is interpolated to N x N (and back). Either pointer may be NULL. */
+int pc_plan_transforms(pc_plan_t plan, int32_t* grid_side, int32_t* image_side);
 int pc_plan_tuning_info(pc_plan_t plan, pc_plan_tuning* out_host);
 /* The part of each w-plane's grid that visibilities can reach (the gridding,
  * the FFT's first pass and the degridding touch nothing else): the number of

@@ -33,6 +33,7 @@ EXPORTS = [
     "pc_profile_begin_classes", "pc_server_create", "pc_server_submit", "pc_server_wait",
     "pc_server_destroy", "pc_plan_tuning_info", "pc_dict_adjoint", "pc_dict_forward_sparse",
     "pc_dict_lambda_max", "pc_solve_synthesis", "pc_forward_grid", "pc_trim_memory", "pc_plan_reach",
+    "pc_plan_transforms",
 ]
 
 
@@ -149,6 +150,7 @@ def load(path: str | None = None):
         "pc_plan_destroy": (None, [_P]),
         "pc_plan_tuning_info": (_I32, [_P, ctypes.POINTER(pc_plan_tuning)]),
         "pc_plan_reach": (_I32, [_P, ctypes.POINTER(_I32), ctypes.POINTER(_I32)]),
+        "pc_plan_transforms": (_I32, [_P, ctypes.POINTER(_I32), ctypes.POINTER(_I32)]),
         "pc_plan_info": (_I32, [_P, ctypes.POINTER(_I32), ctypes.POINTER(_I32), ctypes.POINTER(_I32),
                                 ctypes.POINTER(_I64), ctypes.POINTER(_I32), ctypes.POINTER(_D)]),
         "pc_forward_sparse": (_I32, [_P, _P, _P, _I32, _P, _P]),
@@ -262,6 +264,13 @@ def pc_plan_reach(plan: Plan) -> dict:
     r, c = _I32(), _I32()
     _check(load().pc_plan_reach(plan.handle, ctypes.byref(r), ctypes.byref(c)))
     return dict(rows=r.value, col_groups=c.value)
+
+
+def pc_plan_transforms(plan: Plan) -> dict:
+    """Sides of the grid and of the image that the w-planes are transformed on."""
+    g, n = _I32(), _I32()
+    _check(load().pc_plan_transforms(plan.handle, ctypes.byref(g), ctypes.byref(n)))
+    return dict(transform_grid=g.value, transform_image=n.value)
 
 
 def pc_plan_tuning_info(plan: Plan) -> dict:

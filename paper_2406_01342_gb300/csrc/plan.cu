@@ -1246,6 +1246,14 @@ extern "C" int pc_plan_reach(pc_plan_t p, int32_t* rows, int32_t* col_groups) {
   return PC_OK;
 }
 
+extern "C" int pc_plan_transforms(pc_plan_t p, int32_t* grid_side, int32_t* image_side) {
+  clear_error();
+  if (!p) return fail(PC_ERR_INVALID_ARG, "pc_plan_transforms: NULL plan");
+  if (grid_side) *grid_side = p->G;
+  if (image_side) *image_side = p->Nt;
+  return PC_OK;
+}
+
 extern "C" int pc_plan(const double* uvw_dev, int64_t M, int32_t N, double fov_rad,
                        const pc_plan_opts* opts, void* stream, pc_plan_t* plan_out) {
   return pc_plan_create(uvw_dev, M, N, fov_rad, opts, stream, plan_out);
