@@ -214,11 +214,32 @@ def gram_entries(n_new: int, n_act: int) -> float:
     return n_new * (n_act + 1) - n_new * (n_new - 1) / 2.0
 
 
+def plan_info(abi, plan) -> dict:
+    """Plan geometry, with the grid and the image that the w-planes are transformed on."""
+    return dict(abi.pc_plan_info(plan), **abi.pc_plan_transforms(plan))
+
+
+def transform_grid(info) -> int:
+    return info.get("transform_grid", info["grid_side"])
+
+
+def transform_image(info, wl) -> int:
+    return info.get("transform_image", wl.N)
+
+
+def interpolation_bytes(info, wl) -> float:
+    """Bytes of the interpolation between the image and the smaller one that the planes
+    are transformed on: either image once, the rows between the two passes written and
+    read (0 when the transforms run on the image itself)."""
+    Nt, N = transform_image(info, wl), wl.N
+    return 4.0 * (N * N + Nt * Nt + 2.0 * N * Nt) if Nt != N else 0.0
+
+
 def reach_cells(info, reach):
     """Grid cells per w-plane that visibilities can reach (the gridding, the
     first FFT pass and the degridding touch no others)."""
     if not reach:
-        return float(info["grid_side"]) ** 2
+        return float(transform_grid(info)) ** 2
     return float(reach["rows"]) * 32.0 * reach["col_groups"]
 
 
@@ -245,7 +266,7 @@ def gridding_roofline(prof, info, wl, peaks, reach=None):
         return None
     launches, _, total_ms = prof["grid"]
     avg_ms = total_ms / max(launches, 1)
-    G, P = info["grid_side"], info["n_planes"]
+    G, P = transform_grid(info), info["n_planes"]
     b = 20.0 * wl.M + 8.0 * P * reach_cells(info, reach)
     b_full = 20.0 * wl.M + 8.0 * P * G * G
     hbm = peaks.get("hbm_gbs", 6800.0)
@@ -263,7 +284,8 @@ def degridding_leg(abi, torch, plan, wl, info, peaks, steps, l2_flush) -> dict:
     """The forward operator on a dense image by degridding (pc_forward_grid):
     per call, CUDA events on the launching stream, L2 flushed between calls;
     bytes = the N^2 image read + 8 B per visibility written + the grid planes
-    (written by the second FFT pass and read by the interpolation)."""
+    (written by the second FFT pass and read by the interpolation), of the grid that the
+    planes are transformed on."""
     img = torch.randn(wl.N, wl.N, dtype=torch.float32, device=l2_flush.device)
     y = torch.empty(wl.M, dtype=torch.complex64, device=l2_flush.device)
     for _ in range(3):
@@ -290,7 +312,7 @@ def degridding_leg(abi, torch, plan, wl, info, peaks, steps, l2_flush) -> dict:
     stages = abi.pc_profile_end()
     fft_ms = stages["degrid_fft"][2] / n_prof if "degrid_fft" in stages else 0.0
     interp_ms = stages["degrid"][2] / n_prof if "degrid" in stages else 0.0
-    G, P = info["grid_side"], info["n_planes"]
+    G, P = transform_grid(info), info["n_planes"]
     byt = 4.0 * wl.N * wl.N + 8.0 * wl.M + 2 * 8.0 * P * G * G
     hbm = peaks.get("hbm_gbs", 6800.0)
     f = gridding_flops(wl.M, info)
@@ -321,7 +343,7 @@ def roofline(prof, info, wl, history, steps, peaks, dom, reach=None):
     launches = prof[dom][0]
     avg_ms = ms[dom] / max(launches, 1)
     hbm = peaks.get("hbm_gbs", 6800.0)
-    M, N, G, P = wl.M, wl.N, info["grid_side"], info["n_planes"]
+    M, N, G, P = wl.M, transform_image(info, wl), transform_grid(info), info["n_planes"]
     cells = reach_cells(info, reach)
     rows = float(reach["rows"]) if reach else float(G)
     out = {"kernel": dom, "avg_launch_ms": avg_ms, "launches": launches}
@@ -339,13 +361,13 @@ def roofline(prof, info, wl, history, steps, peaks, dom, reach=None):
     elif dom == "degrid_fft":
         # the degridding's two FFT passes: the image read, the reachable grid
         # written, the pass-1 rows written and read
-        b = 4.0 * N * N + 8.0 * P * cells + 2 * 8.0 * P * N * rows
+        b = 4.0 * N * N + 8.0 * P * cells + 2 * 8.0 * P * N * rows + interpolation_bytes(info, wl)
         out.update(bound="hbm", achieved=b / (avg_ms * 1e-3) / 1e9, peak=hbm, unit="GB/s")
     elif dom == "fft_rows":
         b = 8.0 * P * cells + 8.0 * P * N * rows
         out.update(bound="hbm", achieved=b / (avg_ms * 1e-3) / 1e9, peak=hbm, unit="GB/s")
     elif dom == "fft_cols":
-        b = 8.0 * P * N * rows + 16.0 * N * N + 4.0 * N * N
+        b = 8.0 * P * N * rows + 16.0 * N * N + 4.0 * N * N + interpolation_bytes(info, wl)
         out.update(bound="hbm", achieved=b / (avg_ms * 1e-3) / 1e9, peak=hbm, unit="GB/s")
     elif dom == "apgd":
         # one S x S FP32 GEMV per iteration (G read from shared memory or L2)
@@ -657,7 +679,7 @@ def secondary_leg(abi, synth, torch, device, name, steps, l2_flush, peaks) -> di
     breakdown pass, then timed solves (median), the dominant kernel's
     roofline and the plain-FP32 contraction beside the default."""
     wl, _, plan, V = make_inputs(abi, synth, name, device)
-    info = abi.pc_plan_info(plan)
+    info = plan_info(abi, plan)
     reach = abi.pc_plan_reach(plan)
     lmax = abi.pc_lambda_max(plan, V)
     lam = wl.alpha * lmax
@@ -696,7 +718,7 @@ def coplanar_gridding_leg(abi, synth, torch, device, names, l2_flush, peaks, rep
         uvw = wl.uvw.copy()
         uvw[:, 2] = 0.0
         plan = abi.pc_plan_create(torch.from_numpy(uvw).to(device), wl.N, wl.fov)
-        info = abi.pc_plan_info(plan)
+        info = plan_info(abi, plan)
         reach = abi.pc_plan_reach(plan)
         h = torch.from_numpy(wl.noise.astype(np.complex64)).to(device)
         for _ in range(3):
@@ -709,7 +731,8 @@ def coplanar_gridding_leg(abi, synth, torch, device, names, l2_flush, peaks, rep
         prof = abi.pc_profile_end()
         torch.cuda.synchronize()
         out[name + "_coplanar"] = dict(gridding_roofline(prof, info, wl, peaks, reach), n_planes=info["n_planes"],
-                                       grid_side=info["grid_side"], M=wl.M)
+                                       grid_side=info["grid_side"],
+                                       transform_grid=info["transform_grid"], M=wl.M)
         del plan
     return out
 
@@ -726,7 +749,7 @@ def run_ours(args, world, rank, local):
     device = torch.device("cuda", local)
     torch.cuda.set_device(device)
     wl, uvw, plan, V = make_inputs(abi, synth, args.workload, device, autotune=1 if args.autotune else 0)
-    info = abi.pc_plan_info(plan)
+    info = plan_info(abi, plan)
     reach = abi.pc_plan_reach(plan)
     tuning = abi.pc_plan_tuning_info(plan)
     lmax = abi.pc_lambda_max(plan, V)
