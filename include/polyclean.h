@@ -76,9 +76,10 @@ typedef struct {
   int32_t autotune;       /* 1: time the candidate gridding kernels, gridding sub-problem
                              sizes and FFT kernels on this plan's visibilities and keep
                              the fastest (adds a few ms to plan creation); 0 (default): off */
-  int32_t fft_kernel;     /* FFT passes: 0 (default) one warp per row, in registers, where G
-                             is 512 or 1024, else shared-memory Stockham stages; 1: Stockham
-                             everywhere. The autotuner, when on, chooses per pass instead. */
+  int32_t fft_kernel;     /* FFT passes: 0 (default) one warp per row, in registers, where the
+                             planes' grid has side 512 or 1024, one CTA per row from 2048,
+                             else shared-memory Stockham stages; 1: Stockham everywhere, on the
+                             image's own grid. The autotuner, when on, chooses per pass instead. */
 } pc_plan_opts;
 
 /* What the plan-time autotuner chose (tuned = 0 when it did not run). */

@@ -506,8 +506,8 @@ __device__ __forceinline__ void block_sum_f(float (&v)[K], float (*red)[3][8], i
 // What bounds it: up to 800 atoms the latency of exchange, barriers and sums;
 // beyond, the rows that 16 SMs cannot keep, read from L2. Measured against bulk
 // copies of slices with six barriers an iteration, all rows or none in shared
-// memory, us an iteration before and after: 300 atoms 2.30 and 1.46, 500 2.50 and
-// 1.68, 900 5.5 and 3.8, 1300 7.2 and 5.7, 2500 16.8 and 16.0.
+// memory, us an iteration before and after: 300 atoms 2.30 and 1.56, 500 2.46 and
+// 1.79, 900 5.5 and 3.8, 1300 7.2 and 5.7, 2500 16.8 and 16.0.
 
 constexpr long long APGD_WAIT_CYCLES = 4000000000ll;   // ~2 s at 2 GHz
 
@@ -857,8 +857,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_apgd_full(const __grid_constant_
 // cooperative (all CTAs resident); every wait has a limit.
 //
 // What bounds it: the latency of the exchange. Measured against k_apgd_full on 16
-// SMs, us an iteration: 900 atoms 3.8 and 2.9, 1300 5.7 and 2.8, 1700 8.1 and 3.4,
-// 2500 16.0 and 4.2.
+// SMs, us an iteration: 900 atoms 3.8 and 2.8, 1300 5.7 and 2.7, 1700 8.1 and 3.0,
+// 2500 16.0 and 3.8.
 constexpr int GRID_THREADS = 256;
 constexpr int GRID_EMAX = 12;                       // entries per thread: supports of up to 3072
 constexpr int GRID_ROWS = 32;                       // rows per CTA at most: four a warp (a multiple of 4)
@@ -1099,7 +1099,7 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) k_apgd_grid(const __grid_cons
 // product and the stop test during the next proximal step, which a stop discards.
 // Measured against a thread per row with G in shared memory (and one warp for
 // the whole problem up to 64 atoms), us an iteration before and after: 40 atoms
-// 0.66 and 0.50, 120 1.09 and 0.59, 160 1.31 and 1.03, 224 1.83 and 1.28.
+// 0.66 and 0.50, 120 1.09 and 0.60, 160 1.31 and 1.03, 224 1.83 and 1.28.
 //
 // Order of the sums: a warp holds 16 rows, every second of 32 consecutive ones
 // (SMALL: every fourth of all 64, rows r and r + 32 first), so that the sums over
@@ -1487,7 +1487,7 @@ ApgdArgs make_args(const ApgdJob& j, const ApgdShape& sh) {
 
 // Whole-GPU shape of a support whose G a cluster would read from L2 (cl: its cluster
 // shape): from about 870 atoms, where the cluster is the slower one (us an iteration,
-// 700 atoms 2.5 on the cluster and 2.4, 900 3.8 and 2.9, 1300 5.7 and 2.8), to about
+// 700 atoms 2.5 on the cluster and 2.4, 900 3.8 and 2.8, 1300 5.7 and 2.7), to about
 // 2750, where one CTA per SM no longer holds all rows.
 static bool apgd_grid_shape(int S, const ApgdShape& cl, ApgdShape* sh) {
   if (!cl.full || cl.cta >= 0 || cl.cache >= cl.rows_per || S > GRID_THREADS * GRID_EMAX) return false;

@@ -9,10 +9,13 @@
 // the w-screen and the 1/n factor.
 //
 // Geometry (all in FP64 here, once per plan):
-//   g_u = frac(u dl) G  in [0, G)   grid coordinate in cells (the uv grid is G-periodic)
+//   g_u = frac(u dl) G  in [0, G)   grid coordinate in cells (the uv grid is G-periodic;
+//   dl and G of the image that the planes are transformed on, see choose_resample)
 //   x_w = (w - w0) / dw             plane coordinate
 //   planes p = ceil(x_w - W/2) ... + W - 1, with dw <= 1 / (2 (s_max - s_min)),
-//   s = n - 1 over the image, so that |dw (s - s_c)| <= 1/4 (oversampling 2 in w).
+//   s = n - 1 over that image, so that |dw (s - s_c)| <= 1/4 (oversampling 2 in w) on the N
+//   x N pixels; up to 1/3 on the rim of a smaller image, which only the outer taps of
+//   the interpolation read.
 // Each visibility is replicated into every tile its W x W footprint touches
 // (at most 2 x 2 tiles since W <= T), so a gridding CTA only ever reads the
 // visibilities that touch its own tile.

@@ -960,9 +960,11 @@ int SolveJob::process() {
 // iteration) plus a negligible APGD on G; the operator form costs one
 // degridding + gridding pair per Lanczos step (about 16) and per FISTA
 // iteration (estimated by the previous reweighting's count, at least 20).
-// Contraction rates are the ones measured on this GPU for the kernel the
-// Gram form would use (tensor cores ~0.5 PFLOP/s on split FP16 including the
-// phase generation; FP32 CUDA cores ~24 TFLOP/s on full tiles).
+// Contraction rates are ones measured on this GPU for the kernel the Gram form
+// would use (FP32 CUDA cores ~24 TFLOP/s on full tiles; tensor cores ~0.5 PFLOP/s on
+// split FP16 including the phase generation, which the contraction's present schedule
+// has raised to 0.8 at 1001 atoms x 1M: the choice still counts the former rate, so
+// between the two it takes the operator form early).
 int SolveJob::choose_form(int n_new, int n_act, bool* op) {
   *op = false;
   if (c.reweight == 1 || p->M <= 0) return PC_OK;
